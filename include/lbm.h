@@ -192,7 +192,10 @@ typedef struct {
  * cell list in one launch per time step, a CTA per chunk of up to
  * march_planes planes of a throat, which computes the densities of a plane and steps the plane below
  * it right after (a plane's pairs are read a second time from cache, not from
- * DRAM).  All forms give bit-identical rows.  AUTO is CELLS. */
+ * DRAM).  All forms give bit-identical rows.  AUTO is CELLS, except that with
+ * tau = 1 in both components the throats whose populations fit the shared memory
+ * of one thread-block cluster (up to about 22 000 open cells) run there, all
+ * steps of an increment in one launch. */
 #define LBM_BATCH_AUTO 0
 #define LBM_BATCH_PERSISTENT 1
 #define LBM_BATCH_PER_STEP 2
@@ -251,9 +254,9 @@ int lbm_throat_lattice_features(const double* throats, int n, double* out);
  * n throats at once: each throat's box (lbm_throat_geometry) starts filled with
  * wetting fluid, then runs the schedule's ladder exactly as lbm_run_drainage
  * would on that box alone.  All throats run together in one device arena, in the
- * form sched->batch_form selects (LBM_BATCH_CELLS by default: the throats'
- * non-solid cells as one list, two launches per time step; see the forms
- * above); one increment is captured as a CUDA graph and relaunched.  Every form
+ * form sched->batch_form selects (by default the throats' non-solid cells, on
+ * chip where they fit, else as one list with two launches per time step; see the
+ * forms above); one increment is captured as a CUDA graph and relaunched.  Every form
  * gives the same rows bit for bit.  The host set-up (voxelising the boxes,
  * building the lists) runs on all host cores.
  *   throats   n x 3 x 4 doubles (host)

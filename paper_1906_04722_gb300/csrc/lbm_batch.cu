@@ -1,4 +1,4 @@
-// lbm_batch.cu -- many pore throats per call (lbm_run_throat_batch), in four
+// lbm_batch.cu -- many pore throats per call (lbm_run_throat_batch), in five
 // forms that give the same rows bit for bit.
 //
 // The hybrid method runs one small LBM simulation per pore throat (Sec. 2.2.2)
@@ -6,12 +6,16 @@
 // a batch run together on the GPU, each with its own box, geometry words and
 // reservoir ladder, found through a record table.
 //
-// Cell list (the default).  A throat box is mostly grain: it is the bounding box
+// Cell list.  A throat box is mostly grain: it is the bounding box
 // of a triangular prism whose corners the spheres fill.  This form stores the
 // populations of the non-solid cells only, compactly and after streaming, and
 // runs two launches per time step over that list: densities, then the
 // collision, which pushes every value to the cell it streams to.  A measurement
 // launch (a CTA per slice of a throat box) ends each increment.
+//
+// On chip (lbm_resident.cu; AUTO, tau = 1 in both components).  The same list, a
+// throat's populations in the shared memory of one thread-block cluster for all
+// steps of an increment; what does not fit stays with the cell list.
 //
 // March.  The same cell list in one launch per time step: a CTA per chunk of a
 // throat's planes sums the densities of a plane and steps the plane below it.
@@ -38,6 +42,7 @@
 #include <vector>
 
 #include "lbm_host.h"
+#include "lbm_resident.h"
 #include "lbm_step_core.cuh"
 
 namespace lbmk {
@@ -566,16 +571,17 @@ cudaError_t launch_march(int mt, bool t1, bool nb16, int n_chunks, cudaStream_t 
     return cudaErrorInvalidValue;
 }
 
-// Measurements of the cell-list form from the compact populations, one CTA per
-// slice of a throat box: slice (throat, first box cell, end box cell, index of
+// Measurements of the cell-list form from the compact populations (items below
+// n_list: fc, stride cp; the on-chip form's items from n_list on: fr, stride
+// rp), one CTA per slice of a throat box: slice (throat, first box cell, end box cell, index of
 // the throat's first slice), walked in the box order of the box-layout forms
 // through the box -> item map (the same sums, the same rounding).  The last CTA
 // of a throat to finish adds its slices' sums in slice order and writes the
 // row; the last CTA of all advances the increment index.
 __global__ void __launch_bounds__(BATCH_THREADS)
     cell_measure_kernel(const ThroatRec* __restrict__ recs, const int4* __restrict__ slices, int n_slices,
-                        const int* __restrict__ box_to_item, int cp, const float2* __restrict__ fc,
-                        const uint32_t* __restrict__ wc, double G, const double* __restrict__ rin_all,
+                        const int* __restrict__ box_to_item, int n_list, int cp, const float2* __restrict__ fc,
+                        int rp, const float2* __restrict__ fr, const uint32_t* __restrict__ wc, double G, const double* __restrict__ rin_all,
                         int ladder_stride, lbm_increment* __restrict__ rows, int n_incr, double* partials,
                         int* throat_done, int* incr_now, int* done) {
     __shared__ double red[32];
@@ -592,9 +598,11 @@ __global__ void __launch_bounds__(BATCH_THREADS)
         if (j < 0) return (uint32_t)CLS_SOLID << CLS_SHIFT;
         const uint32_t w = wc[j];
         const uint32_t cls = (w >> CLS_SHIFT) & CLS_MASK;
-        for (int k = 0; k < Q; ++k) rw += fc[(size_t)k * cp + j].x;
+        const float2* f = j < n_list ? fc + j : fr + (j - n_list);
+        const size_t stride = j < n_list ? cp : rp;
+        for (int k = 0; k < Q; ++k) rw += f[k * stride].x;
         if (cls != CLS_MEMBRANE)
-            for (int k = 0; k < Q; ++k) rn += fc[(size_t)k * cp + j].y;
+            for (int k = 0; k < Q; ++k) rn += f[k * stride].y;
         return w;
     };
     double part[NMEAS];
@@ -677,6 +685,136 @@ __global__ void throat_init_kernel(const ThroatRec* __restrict__ recs, int n, fl
             }
         }
     }
+}
+
+// Which throats step on chip (lbm_resident.cu), and how: throats of one shape and
+// cluster size form a class, one launch each.
+struct ResidentPlan {
+    struct Class {
+        int shape, cluster, first, count;
+    };
+    std::vector<ResidentThroat> list;  // class by class
+    std::vector<Class> classes;
+    std::vector<uint8_t> chosen;       // per throat of the batch
+};
+
+// The largest distance in the list between an open cell and one of its 18
+// neighbours (at least: an upper bound from whole rows).
+int list_reach(const std::vector<int>& cells, int ny, int nz) {
+    std::vector<int> row((size_t)ny * nz + 1);
+    size_t j = 0;
+    for (int r = 0; r <= ny * nz; ++r) {
+        while (j < cells.size() && (cells[j] >> 20) * ny + ((cells[j] >> 10) & 1023) < r) ++j;
+        row[(size_t)r] = (int)j;
+    }
+    int reach = 1;
+    for (int r = 0; r < ny * nz; ++r) {
+        const int far = std::min(ny * nz - 1, r + ny + 1);  // row (y + 1, z + 1)
+        if (row[(size_t)r + 1] > row[(size_t)r]) reach = std::max(reach, row[(size_t)far + 1] - 1 - row[(size_t)r]);
+    }
+    return reach;
+}
+
+// Shapes and cluster sizes.  With C CTAs of `per` cells each a step takes about
+// 1.4 + 2.9 per / 1000 us (measured: 1.8 at 140 cells, 2.7 at 440, 4.3 at 1000),
+// and the GPU holds held(C) such clusters at once -- not 152 / C: a cluster lives
+// in one GPC, so that 23 clusters of 6 fit but 15 of 7, 8 or 9 (the kernel's
+// occupancy query says).  Launches of different cluster sizes overlap poorly once
+// a batch takes several rounds, so it takes one base size for every throat that
+// it holds and few larger ones for the rest; a batch that fits the GPU at once
+// rather takes the smallest size for each of the rest.  The base (and which of
+// the two) is the one with the least estimated time.
+struct ResidentBase {
+    int shape, cluster, fine;
+};
+constexpr int RESIDENT_LARGER[][2] = {{0, 9}, {1, 9}, {0, 16}, {1, 16}};  // (shape, cluster)
+
+void plan_resident(const std::vector<std::vector<int>>& cells_of, const std::vector<int>& reach, ResidentPlan& plan) {
+    const int n = (int)cells_of.size();
+    auto per = [&](int t, int c) { return std::max((int)((cells_of[t].size() + c - 1) / c), reach[t]); };
+    auto fits = [&](int t, int s, int c) {
+        return !cells_of[t].empty() && per(t, c) <= resident_cells(s) && reach[t] <= resident_max_reach(s);
+    };
+    ResidentBase best_base = {-1, 0, 0};
+    double best = 1e300;
+    // the class of throat t: the base's, or the first larger one that holds t
+    auto class_of = [&](int t, const ResidentBase& base) -> std::array<int, 2> {
+        if (fits(t, base.shape, base.cluster)) return {base.shape, base.cluster};
+        if (base.fine) {
+            for (int c = base.cluster; c <= RESIDENT_MAX_CLUSTER; ++c)
+                if (resident_clusters(1, c) > 0 && fits(t, 1, c)) return {1, c};
+        } else {
+            for (const auto& l : RESIDENT_LARGER)
+                if (l[1] >= base.cluster && resident_clusters(l[0], l[1]) > 0 && fits(t, l[0], l[1])) return {l[0], l[1]};
+        }
+        return {-1, 0};
+    };
+    static_assert(RESIDENT_SHAPES == 2, "bases: every shape and size, coarse and fine");
+    for (int b = 0; b < 2 * RESIDENT_SHAPES * RESIDENT_MAX_CLUSTER; ++b) {
+        const ResidentBase base = {b % 2, 1 + (b / 2) % RESIDENT_MAX_CLUSTER, b / (2 * RESIDENT_MAX_CLUSTER)};
+        if (resident_clusters(base.shape, base.cluster) < 1) continue;
+        double count[RESIDENT_SHAPES][RESIDENT_MAX_CLUSTER + 1] = {}, us[RESIDENT_SHAPES][RESIDENT_MAX_CLUSTER + 1] = {};
+        double longest = 0.0, share = 0.0, total = 0.0;
+        long long left = 0;  // cells of throats that stay with the cell list
+        for (int t = 0; t < n; ++t) {
+            const std::array<int, 2> k = class_of(t, base);
+            if (k[0] < 0) {
+                left += (long long)cells_of[t].size();
+                continue;
+            }
+            const double step = 1.4 + 2.9e-3 * per(t, k[1]);
+            count[k[0]][k[1]] += 1.0;
+            us[k[0]][k[1]] += step;
+            longest = std::max(longest, step);
+        }
+        for (int i = 0; i < RESIDENT_SHAPES; ++i)
+            for (int j = 1; j <= RESIDENT_MAX_CLUSTER; ++j) {
+                if (count[i][j] == 0.0) continue;
+                const double held = resident_clusters(i, j);
+                share += count[i][j] / held;
+                total += std::ceil(count[i][j] / held) * us[i][j] / count[i][j];
+            }
+        const double est = (share <= 1.0 ? longest : total) + (left ? 12.0 + 80e-6 * (double)left : 0.0);
+        if (est < best) {
+            best = est;
+            best_base = base;
+        }
+    }
+    if (best_base.shape < 0) return;
+    std::vector<std::array<int, 2>> cls((size_t)n);
+    std::vector<int> order;
+    for (int t = 0; t < n; ++t) {
+        cls[t] = class_of(t, best_base);
+        if (cls[t][0] >= 0) order.push_back(t);
+    }
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+        if (cls[a][1] != cls[b][1]) return cls[a][1] > cls[b][1];
+        if (cls[a][0] != cls[b][0]) return cls[a][0] > cls[b][0];
+        return cells_of[a].size() > cells_of[b].size();
+    });
+    for (int t : order) {
+        if (plan.classes.empty() || plan.classes.back().shape != cls[t][0] || plan.classes.back().cluster != cls[t][1])
+            plan.classes.push_back({cls[t][0], cls[t][1], (int)plan.list.size(), 0});
+        ++plan.classes.back().count;
+        plan.list.push_back({0, (int)cells_of[t].size(), reach[t], t});
+        plan.chosen[(size_t)t] = 1;
+    }
+}
+
+// Appends the nodes that the next captured launch of the stream would depend on.
+cudaError_t capture_front(cudaStream_t s, std::vector<cudaGraphNode_t>& nodes) {
+    cudaStreamCaptureStatus st;
+    const cudaGraphNode_t* deps = nullptr;
+    size_t n = 0;
+    cudaError_t e = cudaStreamGetCaptureInfo(s, &st, nullptr, nullptr, &deps, nullptr, &n);
+    if (e == cudaSuccess) nodes.insert(nodes.end(), deps, deps + n);
+    return e;
+}
+
+// Makes the next captured launch of the stream depend on exactly these nodes.
+cudaError_t set_capture_front(cudaStream_t s, std::vector<cudaGraphNode_t>& nodes) {
+    return cudaStreamUpdateCaptureDependencies(s, nodes.data(), nullptr, nodes.size(),
+                                               cudaStreamSetCaptureDependencies);
 }
 
 size_t batch_smem() {
@@ -768,6 +906,9 @@ extern "C" int lbm_run_throat_batch(const double* throats, int n, const lbm_para
             if (rc) return rc;
         }
         std::vector<std::vector<int>> tiles_of((size_t)n), cells_of((size_t)n);
+        std::vector<int> reach((size_t)n);
+        const bool t1 = (float)params->tau[0] == 1.0f && (float)params->tau[1] == 1.0f;
+        const bool try_chip = sched->batch_form == LBM_BATCH_AUTO && t1;
         if (!host_parallel_for(n, [&](int t) {
                 const int nx = dims[t][0], ny = dims[t][1], nz = dims[t][2];
                 const size_t nxy = (size_t)nx * ny;
@@ -786,6 +927,7 @@ extern "C" int lbm_run_throat_batch(const double* throats, int n, const lbm_para
                             for (int x = 0; x < nx; ++x)
                                 if (!(m[(size_t)z * nxy + (size_t)y * nx + x] & LBM_MASK_SOLID))
                                     cl.push_back(x | (y << 10) | (z << 20));
+                    if (try_chip) reach[t] = list_reach(cl, ny, nz);
                     return;
                 }
                 // active tiles: the (30 x 4)-column tiles of the step kernel that
@@ -864,7 +1006,12 @@ extern "C" int lbm_run_throat_batch(const double* throats, int n, const lbm_para
         lbm_increment* d_rows = nullptr;
         cudaGraphExec_t exec = nullptr;
         cudaStream_t cap = nullptr;
+        ResidentBox* d_boxes = nullptr;
+        ResidentThroat* d_chip = nullptr;
+        uint4* d_rows16 = nullptr;
+        float2* ar = nullptr;  // populations of the throats that step on chip
         auto cleanup = [&]() {
+            cudaFree(d_boxes); cudaFree(d_chip); cudaFree(d_rows16); cudaFree(ar);
             cudaFree(a0); cudaFree(a1); cudaFree(d_bc); cudaFree(d_mask); cudaFree(d_nbr); cudaFree(d_nbr_nw);
             cudaFree(d_adh); cudaFree(d_recs); cudaFree(d_order); cudaFree(d_counter); cudaFree(d_rows);
             cudaFree(d_tiles);
@@ -964,13 +1111,22 @@ extern "C" int lbm_run_throat_batch(const double* throats, int n, const lbm_para
         BATCH_CUDA(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
 
         if (cell_list) {
-            // every non-solid cell of every throat (largest throats first,
-            // memory order inside a throat), and the box -> item map
+            // AUTO with tau = 1 in both components: the throats that fit a cluster's
+            // shared memory step on chip, the others by the cell list
+            ResidentPlan plan;
+            plan.chosen.assign((size_t)n, 0);
+            if (try_chip) plan_resident(cells_of, reach, plan);
+            std::stable_partition(order.begin(), order.end(), [&](int t) { return !plan.chosen[(size_t)t]; });
+            // every non-solid cell of every throat (cell-list throats, then on-chip
+            // ones, largest first, memory order inside a throat), and the box ->
+            // item map
             std::vector<long long> item0((size_t)n);
             long long n_items = 0;
+            long long n_listed = 0;
             for (int t : order) {
                 item0[t] = n_items;
                 n_items += (long long)cells_of[t].size();
+                if (!plan.chosen[(size_t)t]) n_listed = n_items;
             }
             if (n_items > (long long)INT_MAX - 64) {
                 cleanup();
@@ -991,8 +1147,9 @@ extern "C" int lbm_run_throat_batch(const double* throats, int n, const lbm_para
                     map[(size_t)(v >> 20) * g.nxy + (size_t)((v >> 10) & 1023) * g.nx + (v & 1023)] = item;
                 }
             });
-            const int n_cells = (int)cells.size();
-            const int cp = (n_cells + 31) / 32 * 32;
+            const int n_cells = (int)n_listed, n_all = (int)cells.size(), n_chip = n_all - n_cells;
+            const int cp = (n_cells + 31) / 32 * 32, rp = (n_chip + 31) / 32 * 32;
+            const int wp = std::max(32, (n_all + 31) / 32 * 32);
             // marching form: the first item of every plane of every throat, and
             // chunks of at most march_planes planes, largest throats first
             int n_chunks = 0;
@@ -1038,7 +1195,7 @@ extern "C" int lbm_run_throat_batch(const double* throats, int n, const lbm_para
             BATCH_CUDA(cudaMalloc(&d_cells, sizeof(int2) * std::max<size_t>(1, cells.size())));
             BATCH_CUDA(cudaMalloc(&d_map, sizeof(int) * (size_t)std::max<long long>(1, c_tot)));
             BATCH_CUDA(cudaMalloc(&d_rho2, sizeof(float2) * (size_t)std::max(cp, 32)));
-            BATCH_CUDA(cudaMalloc(&d_wc, sizeof(uint32_t) * 3 * (size_t)std::max(cp, 32)));
+            BATCH_CUDA(cudaMalloc(&d_wc, sizeof(uint32_t) * 3 * (size_t)wp));
             // 16-bit push-table offsets where every throat's neighbours lie within reach
             long long reach = 0;
             for (const ThroatRec& r : recs) reach = std::max(reach, (long long)r.g.nxy + r.g.nx + 1);
@@ -1048,15 +1205,16 @@ extern "C" int lbm_run_throat_batch(const double* throats, int n, const lbm_para
             BATCH_CUDA(cudaMalloc(&a1, sizeof(float) * fc_floats));
             BATCH_CUDA(cudaMalloc(&d_incr, sizeof(int) * 2));
             BATCH_CUDA(cudaMemsetAsync(d_incr, 0, sizeof(int) * 2, stream));
-            uint32_t* d_wnc = d_wc + std::max(cp, 32);
-            uint32_t* d_adhc = d_wnc + std::max(cp, 32);
+            uint32_t* d_wnc = d_wc + wp;
+            uint32_t* d_adhc = d_wnc + wp;
             if (c_tot)
                 BATCH_CUDA(cudaMemcpyAsync(d_map, box_to_item.data(), sizeof(int) * box_to_item.size(),
                                            cudaMemcpyHostToDevice, stream));
             const unsigned blocks = (unsigned)((n_cells + CELL_THREADS - 1) / CELL_THREADS);
-            if (n_cells) {
+            if (n_all)
                 BATCH_CUDA(cudaMemcpyAsync(d_cells, cells.data(), sizeof(int2) * cells.size(), cudaMemcpyHostToDevice,
                                            stream));
+            if (n_cells) {
                 if (nb16)
                     cell_gather_kernel<int16_t><<<blocks, CELL_THREADS, 0, stream>>>(
                         d_recs, d_cells, n_cells, cp, d_nbr, d_nbr_nw, d_adh, d_map, d_wc, d_wnc, d_adhc,
@@ -1071,6 +1229,27 @@ extern "C" int lbm_run_throat_batch(const double* throats, int n, const lbm_para
                                                                      (float)params->rho_minor);
                 BATCH_CUDA(cudaGetLastError());
             }
+            std::vector<ResidentBox> boxes;
+            if (n_chip) {
+                for (int t = 0; t < n; ++t) {
+                    const Geom& g = recs[t].g;
+                    boxes.push_back({recs[t].c_off, g.nx, g.ny, g.nz, (int)item0[t]});
+                }
+                for (ResidentThroat& th : plan.list) th.item0 = (int)(item0[th.id] - n_listed);
+                BATCH_CUDA(cudaMalloc(&d_boxes, sizeof(ResidentBox) * (size_t)n));
+                BATCH_CUDA(cudaMalloc(&d_chip, sizeof(ResidentThroat) * plan.list.size()));
+                BATCH_CUDA(cudaMalloc(&d_rows16, sizeof(uint4) * (size_t)rp));
+                BATCH_CUDA(cudaMalloc(&ar, sizeof(float2) * Q * (size_t)rp));
+                BATCH_CUDA(cudaMemcpyAsync(d_boxes, boxes.data(), sizeof(ResidentBox) * (size_t)n,
+                                           cudaMemcpyHostToDevice, stream));
+                BATCH_CUDA(cudaMemcpyAsync(d_chip, plan.list.data(), sizeof(ResidentThroat) * plan.list.size(),
+                                           cudaMemcpyHostToDevice, stream));
+                BATCH_CUDA(launch_resident_rows(d_cells, n_cells, n_all, d_boxes, d_map, d_nbr, d_adh, d_wc, d_adhc,
+                                                d_rows16, stream));
+                cell_init_kernel<<<(unsigned)((n_chip + CELL_THREADS - 1) / CELL_THREADS), CELL_THREADS, 0, stream>>>(
+                    d_wc + n_cells, n_chip, rp, ar, (float)params->rho_major, (float)params->rho_minor);
+                BATCH_CUDA(cudaGetLastError());
+            }
             BATCH_CUDA(cudaStreamSynchronize(stream));  // host lists go out of scope
             const int n_graphs = (sched->n_steps & 1) ? 2 : 1;
             for (int gi = 0; gi < n_graphs; ++gi) {
@@ -1080,7 +1259,6 @@ extern "C" int lbm_run_throat_batch(const double* throats, int n, const lbm_para
                     const int c = (gi + st) & 1;
                     const float2* fin = reinterpret_cast<const float2*>(c ? a1 : a0);
                     float2* fout = reinterpret_cast<float2*>(c ? a0 : a1);
-                    const bool t1 = P.tau[0] == 1.0f && P.tau[1] == 1.0f;
                     const int ls = sched->per_throat ? I : 0;
                     const int16_t* nb16p = static_cast<const int16_t*>(d_nbp);
                     const int* nb32p = static_cast<const int*>(d_nbp);
@@ -1110,10 +1288,28 @@ extern "C" int lbm_run_throat_batch(const double* throats, int n, const lbm_para
                             d_cells, n_cells, cp, fin, fout, d_rho2, d_wc, d_wnc, d_adhc, nb32p, P, d_bc, ls, d_incr);
                     cerr = cudaGetLastError();
                 }
+                // the on-chip classes: one launch each for all steps, side by side, after
+                // the cell list's steps (beside them, every short launch of the list
+                // would wait for an SM that a cluster holds for all of the increment)
+                // in the graph: each class depends on what came before all of them,
+                // the measurement on every class
+                std::vector<cudaGraphNode_t> before, after;
+                if (n_chip && cerr == cudaSuccess) cerr = capture_front(cap, before);
+                for (size_t c = 0; c < plan.classes.size() && cerr == cudaSuccess; ++c) {
+                    const ResidentPlan::Class& k = plan.classes[c];
+                    cerr = set_capture_front(cap, before);
+                    if (cerr == cudaSuccess)
+                        cerr = launch_resident(k.shape, k.cluster, k.count, d_chip + k.first, ar, ar, rp,
+                                               d_wc + n_cells, d_adhc + n_cells, d_rows16, P, d_bc,
+                                               sched->per_throat ? I : 0, d_incr, sched->n_steps, (int)c, cap);
+                    if (cerr == cudaSuccess) cerr = capture_front(cap, after);
+                }
+                if (n_chip && cerr == cudaSuccess) cerr = set_capture_front(cap, after);
                 if (cerr == cudaSuccess) {
                     const int c = (gi + sched->n_steps) & 1;
                     cell_measure_kernel<<<n_slices, dim3(32, BATCH_BY), 0, cap>>>(
-                        d_recs, d_slices, n_slices, d_map, cp, reinterpret_cast<const float2*>(c ? a1 : a0), d_wc,
+                        d_recs, d_slices, n_slices, d_map, n_cells, cp, reinterpret_cast<const float2*>(c ? a1 : a0),
+                        rp, ar, d_wc,
                         params->G, d_rin, sched->per_throat ? I : 0, d_rows, I, d_partials, d_throat_done, d_incr,
                         d_incr + 1);
                     cerr = cudaGetLastError();
