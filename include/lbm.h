@@ -612,8 +612,8 @@ int lbm_get_tile(const lbm_domain* d, int* by, int* lz, int* lead);
  *                      densities; one box load of the words and one of the
  *                      density pairs per plane (boxes without periodic x or y
  *                      and with nx % 4 == 0).  Its results equal the staged
- *                      16-bit kernel's bit for bit; the read-outs convert a
- *                      copy into the pull layout.
+ *                      16-bit kernel's bit for bit; the read-outs read
+ *                      either layout.
  * New domains use LBM_KERNEL_STAGED (lbm_autotune times every kind that applies
  * on the domain).  All give the same results up to rounding (not bit for bit:
  * the TMA kernel folds omega w_k into its equilibrium constants).  LBM_ERR_ARG

@@ -174,21 +174,6 @@ int pull_view(lbm_domain* d, const float** out) {
     return LBM_OK;
 }
 
-// The current 16-bit words in the pull layout, for the read-out kernels: f[cur]
-// itself, or (push layout) their conversion into the other buffer, which the
-// next step overwrites anyway.  The density pairs are R[cur] either way.
-int pull16_view(lbm_domain* d, const uint32_t** out) {
-    const uint32_t* in = reinterpret_cast<const uint32_t*>(d->f[d->cur]);
-    if (d->layout == 0) {
-        *out = in;
-        return LBM_OK;
-    }
-    uint32_t* o = reinterpret_cast<uint32_t*>(d->f[d->cur ^ 1]);
-    LBM_CUDA(launch_push16_to_pull16(in, o, d->d_nbr, d->d_nbr_nw, d->geom, d->stream));
-    *out = o;
-    return LBM_OK;
-}
-
 // Tensor maps of the 16-bit words and density pairs of both buffers for the
 // 16-bit push kernel's current shape.
 int ensure_push16_maps(lbm_domain* d) {
@@ -569,10 +554,8 @@ int lbm_get_density_at(lbm_domain* d, int x, int y, int z, double rho_out[2]) {
         LBM_CUDA(launch_probe(d->f[d->cur], d->d_nbr, d->d_nbr_nw, d->geom, x, y, z, d->d_probe, d->stream));
     }
     else {
-        const uint32_t* w16 = nullptr;
-        if (int rc = pull16_view(d, &w16)) return rc;
-        LBM_CUDA(launch_probe16(d->params.precision, w16, d->R[d->cur],
-                                d->d_nbr, d->d_nbr_nw, d->geom, x, y, z, d->d_probe, d->stream));
+        LBM_CUDA(launch_probe16(d->params.precision, reinterpret_cast<const uint32_t*>(d->f[d->cur]), d->R[d->cur],
+                                d->d_nbr, d->d_nbr_nw, d->geom, d->layout == 1, x, y, z, d->d_probe, d->stream));
     }
     LBM_CUDA(cudaMemcpyAsync(d->h_result, d->d_probe, sizeof(float) * 2, cudaMemcpyDeviceToHost, d->stream));
     int rc = wait_domain(d);
@@ -636,11 +619,9 @@ int lbm_measure(lbm_domain* d, lbm_measurement* out) {
                                 d->meas_blocks, d->d_result, d->stream));
     }
     else {
-        const uint32_t* w16 = nullptr;
-        if (int rc = pull16_view(d, &w16)) return rc;
-        LBM_CUDA(launch_measure16(d->params.precision, w16, d->R[d->cur],
-                                  d->d_nbr, d->d_nbr_nw, d->geom, d->params.G, d->d_partials, d->meas_blocks,
-                                  d->d_result, d->stream));
+        LBM_CUDA(launch_measure16(d->params.precision, reinterpret_cast<const uint32_t*>(d->f[d->cur]), d->R[d->cur],
+                                  d->d_nbr, d->d_nbr_nw, d->geom, d->layout == 1, d->params.G, d->d_partials,
+                                  d->meas_blocks, d->d_result, d->stream));
     }
     LBM_CUDA(cudaMemcpyAsync(d->h_result, d->d_result, sizeof(double) * NMEAS, cudaMemcpyDeviceToHost, d->stream));
     int rc = wait_domain(d);
@@ -682,10 +663,9 @@ int lbm_get_density(lbm_domain* d, double* rho_out) {
             LBM_CUDA(launch_density(d->f[d->cur], d->d_rho, d->d_nbr, d->d_nbr_nw, d->geom, d->stream));
         }
         else {
-            const uint32_t* w16 = nullptr;
-            if (int rc = pull16_view(d, &w16)) return rc;
-            LBM_CUDA(launch_density16(d->params.precision, w16,
-                                      d->R[d->cur], d->d_nbr, d->d_nbr_nw, d->geom, d->d_rho, d->stream));
+            LBM_CUDA(launch_density16(d->params.precision, reinterpret_cast<const uint32_t*>(d->f[d->cur]),
+                                      d->R[d->cur], d->d_nbr, d->d_nbr_nw, d->geom, d->layout == 1, d->d_rho,
+                                      d->stream));
         }
         std::vector<float> tmp((size_t)(2 * d->N));
         LBM_CUDA(cudaMemcpyAsync(tmp.data(), d->d_rho, sizeof(float) * 2 * d->N, cudaMemcpyDeviceToHost, d->stream));

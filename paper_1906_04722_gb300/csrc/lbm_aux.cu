@@ -6,63 +6,12 @@ namespace lbmk {
 
 namespace {
 
-__device__ __forceinline__ bool fluid_w(uint8_t m) { return !(m & LBM_MASK_SOLID); }
-__device__ __forceinline__ bool fluid_nw(uint8_t m) { return !(m & (LBM_MASK_SOLID | LBM_MASK_MEMBRANE)); }
-
-// Geometry words (layout in lbm_internal.h).  For every direction k the pull
-// source x - e_k decides the bounce bit of each component; the neighbour
-// x + e_k contributes 36 w_k e_k to the adhesion vector when it is grain.
 // One thread per cell: x and y from the block and thread, z from blockIdx.z.
 __global__ void __launch_bounds__(256) geometry_kernel(const uint8_t* __restrict__ mask, uint32_t* __restrict__ nbr,
                                                        uint32_t* __restrict__ nbr_nw, uint32_t* __restrict__ adh,
                                                        Geom g) {
     const int x = blockIdx.x * 32 + threadIdx.x, y = blockIdx.y * 8 + threadIdx.y, z = blockIdx.z;
-    if (x >= g.nx || y >= g.ny) return;
-    {
-        const long long c = (long long)z * g.nxy + (long long)y * g.nx + x;
-        const uint8_t m = __ldg(mask + c);
-        uint32_t cls;
-        if (m & LBM_MASK_SOLID) cls = CLS_SOLID;
-        else if (m & LBM_MASK_INLET) cls = CLS_INLET;
-        else if (m & LBM_MASK_OUTLET) cls = CLS_OUTLET;
-        else if (m & LBM_MASK_MEMBRANE) cls = CLS_MEMBRANE;
-        else cls = CLS_FLUID;
-        uint32_t bw = 0, bn = 0;
-        int ax = 0, ay = 0, az = 0;
-        for (int k = 1; k < Q; ++k) {
-            bool ok = true;
-            const int sx = wrap1(x - EX(k), g.nx, g.px, ok);
-            const int sy = wrap1(y - EY(k), g.ny, g.py, ok);
-            const int sz = wrap1(z - EZ(k), g.nz, g.pz, ok);
-            if (!ok) {
-                bw |= 1u << k;
-                bn |= 1u << k;
-            } else {
-                const uint8_t ms = __ldg(mask + (long long)sz * g.nxy + (long long)sy * g.nx + sx);
-                if (!fluid_w(ms)) bw |= 1u << k;
-                if (!fluid_nw(ms)) bn |= 1u << k;
-            }
-            bool ok2 = true;
-            const int tx = wrap1(x + EX(k), g.nx, g.px, ok2);
-            const int ty = wrap1(y + EY(k), g.ny, g.py, ok2);
-            const int tz = wrap1(z + EZ(k), g.nz, g.pz, ok2);
-            if (ok2) {
-                const uint8_t mt = __ldg(mask + (long long)tz * g.nxy + (long long)ty * g.nx + tx);
-                if ((mt & LBM_MASK_SOLID) && (mt & LBM_MASK_ADHESIVE)) {
-                    ax += W36(k) * EX(k);
-                    ay += W36(k) * EY(k);
-                    az += W36(k) * EZ(k);
-                }
-            }
-        }
-        uint32_t word = bw | (cls << CLS_SHIFT);
-        if (bn != bw) word |= BIT_NW_DIFF;
-        if (ax || ay || az) word |= BIT_ADH;
-        nbr[c] = word;
-        nbr_nw[c] = bn;
-        adh[c] = (uint32_t)(uint8_t)(int8_t)ax | ((uint32_t)(uint8_t)(int8_t)ay << 8) |
-                 ((uint32_t)(uint8_t)(int8_t)az << 16);
-    }
+    if (x < g.nx && y < g.ny) geometry_cell(mask, nbr, nbr_nw, adh, g, x, y, z);
 }
 
 // Stored populations whose pull yields the rest equilibrium w_k rho0(x) at every
@@ -128,12 +77,6 @@ __global__ void density_kernel(const float* __restrict__ f, float* __restrict__ 
     }
 }
 
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
 constexpr int MEAS_THREADS = 256;
 
 // Measurements of the current state (definitions in lbm.h), one FP64 partial
@@ -142,9 +85,7 @@ __global__ void __launch_bounds__(MEAS_THREADS) measure_kernel(const float* __re
                                                                const uint32_t* __restrict__ nbr,
                                                                const uint32_t* __restrict__ nbr_nw, Geom g,
                                                                double G, double* __restrict__ partials) {
-    double acc[NMEAS];
-#pragma unroll
-    for (int i = 0; i < NMEAS; ++i) acc[i] = 0.0;
+    MeasureSums sums;
     const long long N = (long long)g.nxy * g.nz;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
         const int ci = (int)c;  // a domain holds fewer than 2^31 cells (lbm_create_domain)
@@ -153,31 +94,29 @@ __global__ void __launch_bounds__(MEAS_THREADS) measure_kernel(const float* __re
         const int z = ci / g.nxy;
         Column col = make_column(x, y, g);
         float dummy[2][Q];
-        float rwf, rnf;
+        float rw, rn;
         int cell;
-        const uint32_t w = pull_cell<false>(f, nbr, nbr_nw, g, col, z, dummy, rwf, rnf, cell);
-        measure_accumulate(acc, (w >> CLS_SHIFT) & CLS_MASK, (double)rwf, (double)rnf, G);
+        const uint32_t w = pull_cell<false>(f, nbr, nbr_nw, g, col, z, dummy, rw, rn, cell);
+        sums.add((w >> CLS_SHIFT) & CLS_MASK, rw, rn, G);
     }
-    __shared__ double red[MEAS_THREADS / 32][NMEAS];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < NMEAS; ++i) {
-        const double v = warp_sum(acc[i]);
-        if (lane == 0) red[wid][i] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < NMEAS) {
-        double v = 0.0;
-        for (int wv = 0; wv < MEAS_THREADS / 32; ++wv) v += red[wv][threadIdx.x];
-        partials[(size_t)blockIdx.x * NMEAS + threadIdx.x] = v;
-    }
+    sums.store<MEAS_THREADS / 32>(partials + (size_t)blockIdx.x * NMEAS);
 }
 
-__global__ void finalize_kernel(const double* __restrict__ partials, int nblocks, double* __restrict__ result) {
-    const int i = threadIdx.x;
-    if (i < NMEAS) {
-        double v = 0.0;
-        for (int b = 0; b < nblocks; ++b) v += partials[(size_t)b * NMEAS + i];
+// The blocks' partials added up: FIN_ROWS threads per sum, each over every
+// FIN_ROWS-th block, then those in order (a single chain over 1216 blocks took
+// 92 us).
+constexpr int FIN_ROWS = 32;
+__global__ void __launch_bounds__(FIN_ROWS* NMEAS)
+    finalize_kernel(const double* __restrict__ partials, int nblocks, double* __restrict__ result) {
+    __shared__ double part[FIN_ROWS][NMEAS];
+    const int i = threadIdx.x % NMEAS, r = threadIdx.x / NMEAS;
+    double v = 0.0;
+#pragma unroll 4
+    for (int b = r; b < nblocks; b += FIN_ROWS) v += partials[(size_t)b * NMEAS + i];
+    part[r][i] = v;
+    __syncthreads();
+    if (r == 0) {
+        for (int q = 1; q < FIN_ROWS; ++q) v += part[q][i];
         result[i] = v;
     }
 }
@@ -221,13 +160,14 @@ cudaError_t launch_density(const float* f, float* rho, const uint32_t* nbr, cons
 }
 
 cudaError_t launch_finalize(const double* partials, int nblocks, double* result, cudaStream_t s) {
-    finalize_kernel<<<1, 32, 0, s>>>(partials, nblocks, result);
+    finalize_kernel<<<1, FIN_ROWS * NMEAS, 0, s>>>(partials, nblocks, result);
     return cudaGetLastError();
 }
 
+// One cell a thread until the GPU is full: a throat-sized box is latency alone.
 int measure_blocks(const Geom& g) {
     const long long N = (long long)g.nxy * g.nz;
-    long long b = (N + MEAS_THREADS * 8 - 1) / (MEAS_THREADS * 8);
+    long long b = (N + MEAS_THREADS - 1) / MEAS_THREADS;
     const long long cap = 8LL * device_sm_count();
     if (b > cap) b = cap;
     if (b < 1) b = 1;
@@ -239,8 +179,7 @@ cudaError_t launch_measure(const float* f, const uint32_t* nbr, const uint32_t* 
     measure_kernel<<<nblocks, MEAS_THREADS, 0, s>>>(f, nbr, nbr_nw, g, G, partials);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    finalize_kernel<<<1, 32, 0, s>>>(partials, nblocks, result);
-    return cudaGetLastError();
+    return launch_finalize(partials, nblocks, result, s);
 }
 
 }  // namespace lbmk

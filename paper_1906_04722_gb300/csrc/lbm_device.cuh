@@ -126,30 +126,137 @@ __device__ __forceinline__ uint32_t pull_cell(const float* __restrict__ fin, con
     return w;
 }
 
-// Adds one cell's contribution to the measurement sums (definitions in lbm.h):
-// mass and sanity per component where it is fluid, Eq. 5 pressure, reservoir
-// means, interior counts and bulk-phase pressures.
-__device__ __forceinline__ void measure_accumulate(double (&acc)[NMEAS], uint32_t cls, double rw, double rn,
-                                                   double G) {
-    if (cls == CLS_SOLID || cls == CLS_OUTSIDE) return;
-    acc[MS_MASS_W] += rw;
-    if (!isfinite(rw)) acc[MS_N_NONFINITE] += 1.0;
-    else if (rw < 0.0) acc[MS_N_NEGATIVE] += 1.0;
-    if (cls != CLS_MEMBRANE) {
-        acc[MS_MASS_NW] += rn;
-        if (!isfinite(rn)) acc[MS_N_NONFINITE] += 1.0;
-        else if (rn < 0.0) acc[MS_N_NEGATIVE] += 1.0;
+__device__ __forceinline__ bool fluid_w(uint8_t m) { return !(m & LBM_MASK_SOLID); }
+__device__ __forceinline__ bool fluid_nw(uint8_t m) { return !(m & (LBM_MASK_SOLID | LBM_MASK_MEMBRANE)); }
+
+// Geometry words (layout in lbm_internal.h) of cell (x, y, z).  For every
+// direction k the pull source x - e_k decides the bounce bit of each component;
+// the neighbour x + e_k contributes 36 w_k e_k to the adhesion vector when it is
+// grain.
+__device__ __forceinline__ void geometry_cell(const uint8_t* __restrict__ mask, uint32_t* __restrict__ nbr,
+                                              uint32_t* __restrict__ nbr_nw, uint32_t* __restrict__ adh,
+                                              const Geom& g, int x, int y, int z) {
+    const long long c = (long long)z * g.nxy + (long long)y * g.nx + x;
+    const uint8_t m = __ldg(mask + c);
+    uint32_t cls;
+    if (m & LBM_MASK_SOLID) cls = CLS_SOLID;
+    else if (m & LBM_MASK_INLET) cls = CLS_INLET;
+    else if (m & LBM_MASK_OUTLET) cls = CLS_OUTLET;
+    else if (m & LBM_MASK_MEMBRANE) cls = CLS_MEMBRANE;
+    else cls = CLS_FLUID;
+    uint32_t bw = 0, bn = 0;
+    int ax = 0, ay = 0, az = 0;
+#pragma unroll
+    for (int k = 1; k < Q; ++k) {
+        bool ok = true;
+        const int sx = wrap1(x - EX(k), g.nx, g.px, ok);
+        const int sy = wrap1(y - EY(k), g.ny, g.py, ok);
+        const int sz = wrap1(z - EZ(k), g.nz, g.pz, ok);
+        if (!ok) {
+            bw |= 1u << k;
+            bn |= 1u << k;
+        } else {
+            const uint8_t ms = __ldg(mask + (long long)sz * g.nxy + (long long)sy * g.nx + sx);
+            if (!fluid_w(ms)) bw |= 1u << k;
+            if (!fluid_nw(ms)) bn |= 1u << k;
+        }
+        bool ok2 = true;
+        const int tx = wrap1(x + EX(k), g.nx, g.px, ok2);
+        const int ty = wrap1(y + EY(k), g.ny, g.py, ok2);
+        const int tz = wrap1(z + EZ(k), g.nz, g.pz, ok2);
+        if (ok2) {
+            const uint8_t mt = __ldg(mask + (long long)tz * g.nxy + (long long)ty * g.nx + tx);
+            if ((mt & LBM_MASK_SOLID) && (mt & LBM_MASK_ADHESIVE)) {
+                ax += W36(k) * EX(k);
+                ay += W36(k) * EY(k);
+                az += W36(k) * EZ(k);
+            }
+        }
     }
-    const double p = (rw + rn) / 3.0 + G * rw * rn / 3.0;  // Eq. 5
-    if (cls == CLS_INLET) { acc[MS_PIN] += p; acc[MS_N_IN] += 1.0; return; }
-    if (cls == CLS_OUTLET) { acc[MS_POUT] += p; acc[MS_N_OUT] += 1.0; return; }
-    if (cls == CLS_MEMBRANE) return;
-    acc[MS_N_FLUID] += 1.0;
-    if (rw > rn) acc[MS_N_W] += 1.0;
-    const double phi = (rw - rn) / (rw + rn);
-    if (fabs(phi) < 0.5) acc[MS_N_INTERFACE] += 1.0;
-    if (phi > 0.9) { acc[MS_PW] += p; acc[MS_N_BULK_W] += 1.0; }
-    if (phi < -0.9) { acc[MS_PNW] += p; acc[MS_N_BULK_NW] += 1.0; }
+    uint32_t word = bw | (cls << CLS_SHIFT);
+    if (bn != bw) word |= BIT_NW_DIFF;
+    if (ax || ay || az) word |= BIT_ADH;
+    nbr[c] = word;
+    nbr_nw[c] = bn;
+    adh[c] = (uint32_t)(uint8_t)(int8_t)ax | ((uint32_t)(uint8_t)(int8_t)ay << 8) |
+             ((uint32_t)(uint8_t)(int8_t)az << 16);
 }
+
+// A thread's measurement sums (definitions in lbm.h).  GB300 has little FP64
+// throughput, and a division there is some twenty FP64 instructions: the sums
+// that need 64 bits (masses and Eq. 5 pressures) take eight FP64 instructions a
+// cell, the counts are integers, and the phase of a cell is decided in FP32 where
+// that is exact or far from the threshold (with divisions and FP64 counts the
+// 192^3 sample took 0.72 ms a measurement; 0.12 ms is its HBM floor).
+struct MeasureSums {
+    double mass[2] = {0.0, 0.0};
+    double p[4] = {0.0, 0.0, 0.0, 0.0};  // 3 x Eq. 5: bulk wetting, bulk non-wetting, inlet, outlet
+    unsigned n[9] = {};                  // MS_N_FLUID .. MS_N_NEGATIVE
+
+    __device__ __forceinline__ void count(int i, bool yes) { n[i - MS_N_FLUID] += yes ? 1u : 0u; }
+
+    __device__ __forceinline__ void add(uint32_t cls, float rw, float rn, double G) {
+        if (cls == CLS_SOLID || cls == CLS_OUTSIDE) return;
+        const bool has_nw = cls != CLS_MEMBRANE;
+        const double dw = rw, dn = rn;
+        mass[0] += dw;
+        if (has_nw) mass[1] += dn;
+        const bool fw = isfinite(rw), fn = isfinite(rn);
+        count(MS_N_NONFINITE, !fw);
+        count(MS_N_NONFINITE, has_nw && !fn);
+        count(MS_N_NEGATIVE, fw && rw < 0.f);
+        count(MS_N_NEGATIVE, has_nw && fn && rn < 0.f);
+        if (!has_nw) return;
+        const double p3 = fma(G * dw, dn, dw + dn);
+        if (cls == CLS_INLET) { p[2] += p3; count(MS_N_IN, true); return; }
+        if (cls == CLS_OUTLET) { p[3] += p3; count(MS_N_OUT, true); return; }
+        count(MS_N_FLUID, true);
+        count(MS_N_W, rw > rn);
+        // phi = (rw - rn) / (rw + rn): for a positive sum |phi| < 0.5 is rw < 3 rn and
+        // rn < 3 rw, and the sign of a fused multiply-add is exact; phi > 0.9 is
+        // rw > 19 rn, decided in FP32 unless the two are within 1e-4 of each other
+        const float y = rw + rn, a = fmaf(-19.f, rn, rw), b = fmaf(-19.f, rw, rn), near = 1e-4f * y;
+        if (y > 0.f && y < 1e30f && fabsf(a) > near && fabsf(b) > near) {
+            count(MS_N_INTERFACE, fmaf(3.f, rn, -rw) > 0.f && fmaf(3.f, rw, -rn) > 0.f);
+            count(MS_N_BULK_W, a > 0.f);
+            count(MS_N_BULK_NW, b > 0.f);
+            if (a > 0.f) p[0] += p3;
+            if (b > 0.f) p[1] += p3;
+        } else {
+            const double phi = (dw - dn) / (dw + dn);
+            count(MS_N_INTERFACE, fabs(phi) < 0.5);
+            if (phi > 0.9) { p[0] += p3; count(MS_N_BULK_W, true); }
+            if (phi < -0.9) { p[1] += p3; count(MS_N_BULK_NW, true); }
+        }
+    }
+
+    // The sums of a block of WARPS warps into out[NMEAS] (all threads call it).
+    template <int WARPS>
+    __device__ __forceinline__ void store(double* __restrict__ out) const {
+        __shared__ double red[WARPS][NMEAS];
+        const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+        const double d[6] = {mass[0], mass[1], p[0], p[1], p[2], p[3]};
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            double v = d[i];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+            if (lane == 0) red[wid][i] = i < 2 ? v : v * (1.0 / 3.0);
+        }
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const unsigned v = __reduce_add_sync(0xffffffffu, n[i]);
+            if (lane == 0) red[wid][MS_N_FLUID + i] = (double)v;
+        }
+        if (lane == 0) red[wid][MS_SPARE] = 0.0;
+        __syncthreads();
+        if (tid < NMEAS) {
+            double v = 0.0;
+#pragma unroll
+            for (int w = 0; w < WARPS; ++w) v += red[w][tid];
+            out[tid] = v;
+        }
+    }
+};
 
 }  // namespace lbmk

@@ -121,7 +121,8 @@ cudaError_t launch_set_bc(float* bc, float in_w, float in_nw, float out_w, float
 cudaError_t launch_probe(const float* f, const uint32_t* nbr, const uint32_t* nbr_nw, const Geom& g, int x, int y,
                          int z, float* out, cudaStream_t s);
 cudaError_t launch_finalize(const double* partials, int nblocks, double* result, cudaStream_t s);
-// 16-bit storage (precision 1 = FP16, 2 = BF16 deviations; lbm_step16.cu)
+// 16-bit storage (precision 1 = FP16, 2 = BF16 deviations; lbm_step16.cu); the
+// read-outs take either layout (push: each word at the cell that reads it)
 bool tile16_supported(int by, int lead);
 cudaError_t prepare_step16(int precision, const StepTile& t);
 cudaError_t launch_step16(int precision, const uint32_t* win, uint32_t* wout, const float2* Rin, float2* Rout,
@@ -129,12 +130,13 @@ cudaError_t launch_step16(int precision, const uint32_t* win, uint32_t* wout, co
                           const Phys& p, StepTile t, cudaStream_t s);
 cudaError_t launch_init16(const float* rho0, float2* R, const Geom& g, cudaStream_t s);
 cudaError_t launch_density16(int precision, const uint32_t* w, const float2* R, const uint32_t* nbr,
-                             const uint32_t* nbr_nw, const Geom& g, float* rho, cudaStream_t s);
+                             const uint32_t* nbr_nw, const Geom& g, bool push, float* rho, cudaStream_t s);
 cudaError_t launch_measure16(int precision, const uint32_t* w, const float2* R, const uint32_t* nbr,
-                             const uint32_t* nbr_nw, const Geom& g, double G, double* partials, int nblocks,
+                             const uint32_t* nbr_nw, const Geom& g, bool push, double G, double* partials, int nblocks,
                              double* result, cudaStream_t s);
 cudaError_t launch_probe16(int precision, const uint32_t* w, const float2* R, const uint32_t* nbr,
-                           const uint32_t* nbr_nw, const Geom& g, int x, int y, int z, float* out, cudaStream_t s);
+                           const uint32_t* nbr_nw, const Geom& g, bool push, int x, int y, int z, float* out,
+                           cudaStream_t s);
 StepTile default_tile(const Geom& g);
 bool tile_supported(int by, int lead);
 // TMA step kernel (FP32; no periodic x / y, nx % 4 == 0)

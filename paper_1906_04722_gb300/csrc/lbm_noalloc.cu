@@ -29,12 +29,6 @@ constexpr long long NA_MAX_CELLS = 56LL * 1000 * 1000;  // 32-bit population ind
 // written earlier by the same call, so nothing has to be cleared in between.
 static __device__ __align__(256) double g_noalloc_scratch[(NA_MAX_BLOCKS + 1) * NMEAS];
 
-__device__ __forceinline__ double na_warp_sum(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    return v;
-}
-
 // Fluid-ness of a pull source for component s, from its raw mask bits (as the
 // geometry words decide bounce-back): solid stops both components, membrane
 // stops the non-wetting one.
@@ -59,9 +53,7 @@ __device__ __forceinline__ uint32_t na_class(uint8_t m) {
 __global__ void __launch_bounds__(NA_THREADS) na_measure_kernel(const float* __restrict__ f,
                                                                 const uint8_t* __restrict__ mask, Geom g, double G,
                                                                 double* __restrict__ partials) {
-    double acc[NMEAS];
-#pragma unroll
-    for (int i = 0; i < NMEAS; ++i) acc[i] = 0.0;
+    MeasureSums sums;
     const long long N = (long long)g.nxy * g.nz;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
         const uint8_t m = mask[c];
@@ -92,28 +84,23 @@ __global__ void __launch_bounds__(NA_THREADS) na_measure_kernel(const float* __r
             rho[s] = r;
         }
         // the same accumulation as lbm_measure
-        measure_accumulate(acc, cls, (double)rho[0], (double)rho[1], G);
+        sums.add(cls, rho[0], rho[1], G);
     }
-    __shared__ double red[NA_THREADS / 32][NMEAS];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < NMEAS; ++i) {
-        const double v = na_warp_sum(acc[i]);
-        if (lane == 0) red[wid][i] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < NMEAS) {
-        double v = 0.0;
-        for (int wv = 0; wv < NA_THREADS / 32; ++wv) v += red[wv][threadIdx.x];
-        partials[(size_t)blockIdx.x * NMEAS + threadIdx.x] = v;
-    }
+    sums.store<NA_THREADS / 32>(partials + (size_t)blockIdx.x * NMEAS);
 }
 
-__global__ void na_finalize_kernel(const double* __restrict__ partials, int nblocks, double* __restrict__ result) {
-    const int i = threadIdx.x;
-    if (i < NMEAS) {
-        double v = 0.0;
-        for (int b = 0; b < nblocks; ++b) v += partials[(size_t)b * NMEAS + i];
+constexpr int NA_ROWS = 32;
+__global__ void __launch_bounds__(NA_ROWS* NMEAS)
+    na_finalize_kernel(const double* __restrict__ partials, int nblocks, double* __restrict__ result) {
+    __shared__ double part[NA_ROWS][NMEAS];
+    const int i = threadIdx.x % NMEAS, r = threadIdx.x / NMEAS;
+    double v = 0.0;
+#pragma unroll 4
+    for (int b = r; b < nblocks; b += NA_ROWS) v += partials[(size_t)b * NMEAS + i];
+    part[r][i] = v;
+    __syncthreads();
+    if (r == 0) {
+        for (int q = 1; q < NA_ROWS; ++q) v += part[q][i];
         result[i] = v;
     }
 }
@@ -177,7 +164,7 @@ extern "C" int lbm_measure_state_noalloc(const lbm_params* params, const int box
     na_measure_kernel<<<(int)nb, NA_THREADS, 0, s>>>(f_dev, mask_dev, g, params->G, partials);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) {
-        na_finalize_kernel<<<1, 32, 0, s>>>(partials, (int)nb, result);
+        na_finalize_kernel<<<1, NA_ROWS * NMEAS, 0, s>>>(partials, (int)nb, result);
         e = cudaGetLastError();
     }
     double r[NMEAS];

@@ -85,6 +85,38 @@ __device__ __forceinline__ uint32_t pull16_density(const uint32_t* __restrict__ 
     return w;
 }
 
+// The same from the push layout: a cell's words lie at the cell itself.
+template <class H2>
+__device__ __forceinline__ uint32_t push16_density(const uint32_t* __restrict__ win, const float2* __restrict__ Rin,
+                                                   const uint32_t* __restrict__ nbr, const Geom& g, int cell,
+                                                   float& rw, float& rn) {
+    rw = 0.f;
+    rn = 0.f;
+    const uint32_t w = __ldg(nbr + cell);
+    const uint32_t cls = (w >> CLS_SHIFT) & CLS_MASK;
+    if (cls == CLS_SOLID) return w;
+    const float2 R = __ldg(Rin + cell);
+    float b = 0.f;
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+        const float2 h = Pair<H2>::unpack(__ldg(win + (size_t)k * g.plane + cell));
+        rw += h.x + WK(k) * R.x;
+        b += h.y + WK(k) * R.y;
+    }
+    if (cls != CLS_MEMBRANE) rn = b;
+    return w;
+}
+
+template <class H2, bool PUSH>
+__device__ __forceinline__ uint32_t cell16_density(const uint32_t* __restrict__ win, const float2* __restrict__ Rin,
+                                                   const uint32_t* __restrict__ nbr,
+                                                   const uint32_t* __restrict__ nbr_nw, const Geom& g, int c,
+                                                   float& rw, float& rn) {
+    if constexpr (PUSH) return push16_density<H2>(win, Rin, nbr, g, c, rw, rn);
+    const int x = c % g.nx, y = (c / g.nx) % g.ny, z = c / g.nxy;
+    return pull16_density<H2>(win, Rin, nbr, nbr_nw, g, make_column(x, y, g), z, rw, rn);
+}
+
 template <int BY, int LEAD>
 size_t smem16_bytes() {
     // per thread: (LEAD+1) stages of 19 words + an R pair, the ring pair x 4, words and adhesion x (LEAD+1)
@@ -272,59 +304,41 @@ __global__ void __launch_bounds__(32 * BY, 2)
                                 min(z0 + lz, g.nz), smem16);
 }
 
-template <class H2>
+template <class H2, bool PUSH>
 __global__ void density16_kernel(const uint32_t* __restrict__ win, const float2* __restrict__ Rin,
                                  const uint32_t* __restrict__ nbr, const uint32_t* __restrict__ nbr_nw, Geom g,
                                  float* __restrict__ rho) {
     const long long N = (long long)g.nxy * g.nz;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(c % g.nx), y = (int)((c / g.nx) % g.ny), z = (int)(c / g.nxy);
         float rw, rn;
-        pull16_density<H2>(win, Rin, nbr, nbr_nw, g, make_column(x, y, g), z, rw, rn);
+        cell16_density<H2, PUSH>(win, Rin, nbr, nbr_nw, g, (int)c, rw, rn);
         rho[c] = rw;
         rho[N + c] = rn;
     }
 }
 
-template <class H2>
+template <class H2, bool PUSH>
 __global__ void __launch_bounds__(256) measure16_kernel(const uint32_t* __restrict__ win,
                                                         const float2* __restrict__ Rin,
                                                         const uint32_t* __restrict__ nbr,
                                                         const uint32_t* __restrict__ nbr_nw, Geom g, double G,
                                                         double* __restrict__ partials) {
-    double acc[NMEAS];
-#pragma unroll
-    for (int i = 0; i < NMEAS; ++i) acc[i] = 0.0;
+    MeasureSums sums;
     const long long N = (long long)g.nxy * g.nz;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(c % g.nx), y = (int)((c / g.nx) % g.ny), z = (int)(c / g.nxy);
         float rw, rn;
-        const uint32_t w = pull16_density<H2>(win, Rin, nbr, nbr_nw, g, make_column(x, y, g), z, rw, rn);
-        measure_accumulate(acc, (w >> CLS_SHIFT) & CLS_MASK, (double)rw, (double)rn, G);
+        const uint32_t w = cell16_density<H2, PUSH>(win, Rin, nbr, nbr_nw, g, (int)c, rw, rn);
+        sums.add((w >> CLS_SHIFT) & CLS_MASK, rw, rn, G);
     }
-    __shared__ double red[8][NMEAS];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < NMEAS; ++i) {
-        double v = acc[i];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) red[wid][i] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < NMEAS) {
-        double v = 0.0;
-        for (int wv = 0; wv < 8; ++wv) v += red[wv][threadIdx.x];
-        partials[(size_t)blockIdx.x * NMEAS + threadIdx.x] = v;
-    }
+    sums.store<8>(partials + (size_t)blockIdx.x * NMEAS);
 }
 
-template <class H2>
+template <class H2, bool PUSH>
 __global__ void probe16_kernel(const uint32_t* __restrict__ win, const float2* __restrict__ Rin,
-                               const uint32_t* __restrict__ nbr, const uint32_t* __restrict__ nbr_nw, Geom g, int x,
-                               int y, int z, float* out) {
+                               const uint32_t* __restrict__ nbr, const uint32_t* __restrict__ nbr_nw, Geom g, int c,
+                               float* out) {
     float rw, rn;
-    pull16_density<H2>(win, Rin, nbr, nbr_nw, g, make_column(x, y, g), z, rw, rn);
+    cell16_density<H2, PUSH>(win, Rin, nbr, nbr_nw, g, c, rw, rn);
     out[0] = rw;
     out[1] = rn;
 }
@@ -469,30 +483,36 @@ cudaError_t launch_init16(const float* rho0, float2* R, const Geom& g, cudaStrea
     return cudaGetLastError();
 }
 
+#define LBM_READ16(kernel, grid, block, ...)                                                          \
+    do {                                                                                              \
+        if (precision == 1 && push) kernel<__half2, true><<<grid, block, 0, s>>>(__VA_ARGS__);        \
+        else if (precision == 1) kernel<__half2, false><<<grid, block, 0, s>>>(__VA_ARGS__);          \
+        else if (push) kernel<__nv_bfloat162, true><<<grid, block, 0, s>>>(__VA_ARGS__);              \
+        else kernel<__nv_bfloat162, false><<<grid, block, 0, s>>>(__VA_ARGS__);                       \
+    } while (0)
+
 cudaError_t launch_density16(int precision, const uint32_t* w, const float2* R, const uint32_t* nbr,
-                             const uint32_t* nbr_nw, const Geom& g, float* rho, cudaStream_t s) {
-    const int b = grid_cells((long long)g.nxy * g.nz);
-    if (precision == 1) density16_kernel<__half2><<<b, 256, 0, s>>>(w, R, nbr, nbr_nw, g, rho);
-    else density16_kernel<__nv_bfloat162><<<b, 256, 0, s>>>(w, R, nbr, nbr_nw, g, rho);
+                             const uint32_t* nbr_nw, const Geom& g, bool push, float* rho, cudaStream_t s) {
+    LBM_READ16(density16_kernel, grid_cells((long long)g.nxy * g.nz), 256, w, R, nbr, nbr_nw, g, rho);
     return cudaGetLastError();
 }
 
 cudaError_t launch_measure16(int precision, const uint32_t* w, const float2* R, const uint32_t* nbr,
-                             const uint32_t* nbr_nw, const Geom& g, double G, double* partials, int nblocks,
+                             const uint32_t* nbr_nw, const Geom& g, bool push, double G, double* partials, int nblocks,
                              double* result, cudaStream_t s) {
-    if (precision == 1) measure16_kernel<__half2><<<nblocks, 256, 0, s>>>(w, R, nbr, nbr_nw, g, G, partials);
-    else measure16_kernel<__nv_bfloat162><<<nblocks, 256, 0, s>>>(w, R, nbr, nbr_nw, g, G, partials);
+    LBM_READ16(measure16_kernel, nblocks, 256, w, R, nbr, nbr_nw, g, G, partials);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     return launch_finalize(partials, nblocks, result, s);
 }
 
 cudaError_t launch_probe16(int precision, const uint32_t* w, const float2* R, const uint32_t* nbr,
-                           const uint32_t* nbr_nw, const Geom& g, int x, int y, int z, float* out, cudaStream_t s) {
-    if (precision == 1) probe16_kernel<__half2><<<1, 1, 0, s>>>(w, R, nbr, nbr_nw, g, x, y, z, out);
-    else probe16_kernel<__nv_bfloat162><<<1, 1, 0, s>>>(w, R, nbr, nbr_nw, g, x, y, z, out);
+                           const uint32_t* nbr_nw, const Geom& g, bool push, int x, int y, int z, float* out,
+                           cudaStream_t s) {
+    LBM_READ16(probe16_kernel, 1, 1, w, R, nbr, nbr_nw, g, (z * g.ny + y) * g.nx + x, out);
     return cudaGetLastError();
 }
+#undef LBM_READ16
 
 cudaError_t launch_pull16_to_push16(const uint32_t* win, uint32_t* wout, const uint32_t* nbr, const uint32_t* nbr_nw,
                                     const Geom& g, cudaStream_t s) {

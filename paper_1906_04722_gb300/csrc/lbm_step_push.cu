@@ -404,30 +404,14 @@ constexpr int PUSH_MEAS_THREADS = 256;
 __global__ void __launch_bounds__(PUSH_MEAS_THREADS)
     push_measure_kernel(const float* __restrict__ Fs, const uint32_t* __restrict__ nbr, Geom g, double G,
                         double* __restrict__ partials) {
-    double acc[NMEAS];
-#pragma unroll
-    for (int i = 0; i < NMEAS; ++i) acc[i] = 0.0;
+    MeasureSums sums;
     const long long N = (long long)g.nxy * g.nz;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
         float rw, rn;
         const uint32_t w = push_cell_density(Fs, nbr, g, c, rw, rn);
-        measure_accumulate(acc, (w >> CLS_SHIFT) & CLS_MASK, (double)rw, (double)rn, G);
+        sums.add((w >> CLS_SHIFT) & CLS_MASK, rw, rn, G);
     }
-    __shared__ double red[PUSH_MEAS_THREADS / 32][NMEAS];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < NMEAS; ++i) {
-        double v = acc[i];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) red[wid][i] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x < NMEAS) {
-        double v = 0.0;
-        for (int wv = 0; wv < PUSH_MEAS_THREADS / 32; ++wv) v += red[wv][threadIdx.x];
-        partials[(size_t)blockIdx.x * NMEAS + threadIdx.x] = v;
-    }
+    sums.store<PUSH_MEAS_THREADS / 32>(partials + (size_t)blockIdx.x * NMEAS);
 }
 
 __global__ void push_density_kernel(const float* __restrict__ Fs, const uint32_t* __restrict__ nbr, Geom g,
