@@ -103,8 +103,8 @@ __global__ void __launch_bounds__(MEAS_THREADS) measure_kernel(const float* __re
 }
 
 // The blocks' partials added up: FIN_ROWS threads per sum, each over every
-// FIN_ROWS-th block, then those in order (a single chain over 1216 blocks took
-// 92 us).
+// FIN_ROWS-th block, then those in order (1216 blocks: 92 us as a single
+// chain, 10 us).
 constexpr int FIN_ROWS = 32;
 __global__ void __launch_bounds__(FIN_ROWS* NMEAS)
     finalize_kernel(const double* __restrict__ partials, int nblocks, double* __restrict__ result) {

@@ -29,12 +29,24 @@ namespace lbmk {
 
 namespace {
 
-// A CTA computes a TM x TN tile of C in chunks of TK along K, two chunks in flight.
-constexpr int TM = 128, TN = 64, TK = 64, GEMM_THREADS = 128;
-constexpr int A_TILE = TM * TK * 2, B_TILE = TN * TK * 2;  // bytes, 16-bit operands
-constexpr int STAGE = A_TILE + B_TILE;
-constexpr int GEMM_SMEM = 2 * STAGE + 64;  // two stages, then the barriers and the TMEM address
-constexpr int EPI_LD = 33;                 // padded row of the epilogue's transpose buffer
+// A CTA computes a TM x TN tile of C in chunks of TK along K, two chunks in
+// shared memory and the loads of a third in flight in registers.  Training's
+// GEMMs (256 x 256 x 256 per member) are latency: TN = 32 gives them 16 CTAs a
+// member.  Inference's (thousands of rows) re-read A for every column tile: TN =
+// 256 takes a hidden layer's whole width.  What bounded both was the staging: 4-byte
+// loads, eight in flight, and 2-byte stores.  With 16-byte loads of a whole chunk in
+// flight and 16-byte stores: a training layer forward (5 members) 26.5 -> 8.2 us,
+// backward (three launches, now one) 63 -> 12 us; an inference layer of 16384 rows
+// 110 -> 51 us.
+constexpr int TM = 128, TK = 64, GEMM_THREADS = 256;
+constexpr int TN_SMALL = 32, TN_LARGE = 256;
+constexpr int A_TILE = TM * TK * 2;  // bytes, 16-bit operands
+template <int TN>
+constexpr int STAGE = A_TILE + TN * TK * 2;
+constexpr int EPI_LD = 36;  // padded row of the epilogue's transpose buffer (16-byte aligned rows)
+constexpr int EPI_BYTES = 8 * 32 * EPI_LD * 4;
+template <int TN>  // two stages (reused by the epilogue), then the barriers and the TMEM address
+constexpr int GEMM_SMEM = (2 * STAGE<TN> > EPI_BYTES ? 2 * STAGE<TN> : EPI_BYTES) + 64;
 constexpr float LOSS_SCALE = 1024.f;
 constexpr unsigned long long GEMM_WAIT_NS = 2000000000ull;
 
@@ -63,6 +75,7 @@ struct GemmArgs {
     const float* mask;  // mask[m * ldm + n] > 0 keeps the value (EPI_MASK)
     int ldm;
     int epi;
+    int vecA, vecB, vecC;  // rows may be read (written) as float4: bases, strides and extents are multiples of 4
     // per ensemble member (grid z): element offsets of A, B, C, bias, mask
     long long zA, zB, zC, zBias, zMask;
     int* err;                    // set to 1 when a wait for the tensor cores ran out
@@ -115,32 +128,77 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity,
     }
 }
 
-// Stage rows [r0, r0 + R) x columns [k0, k0 + TK) of X(r, k) = X[r * sr + k * sk]
-// (zero outside rows x K) as 16-bit values into a core-matrix tile.  Consecutive
-// threads walk whichever index is contiguous in memory; each thread issues eight
-// loads before it converts and stores any of them.
-template <class T, int R>
-__device__ __forceinline__ void stage_tile(unsigned char* __restrict__ dst, const float* __restrict__ X, int sr,
-                                           int sk, int r0, int rows, int k0, int K, int tid) {
-    constexpr int PER = R * TK / GEMM_THREADS;
-    static_assert(PER % 8 == 0, "tile elements per thread");
-    const bool k_fast = sk == 1;
-#pragma unroll 1
-    for (int j0 = 0; j0 < PER; j0 += 8) {
-        float v[8];
-        int off[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int i = tid + (j0 + j) * GEMM_THREADS;
-            const int r = k_fast ? i / TK : i % R, k = k_fast ? i % TK : i / R;
-            const int gr = r0 + r, gk = k0 + k;
-            off[j] = core_offset(r, k);
-            v[j] = (gr < rows && gk < K) ? __ldg(X + (size_t)gr * sr + (size_t)gk * sk) : 0.f;
+// Rows [r0, r0 + R) x columns [k0, k0 + TK) of X(r, k) (zero outside rows x K) as
+// a 16-bit core-matrix tile: load() issues a thread's global loads, store()
+// rounds and stores them.  KF: k is the contiguous index; a task is 8 columns of
+// a row (one 16-byte store).  Otherwise r is; a task is 4 rows of 8 columns (eight
+// loads along r, four 16-byte stores).  ld: the other index's stride.
+template <class T, int R, bool KF>
+struct Tile {
+    static constexpr int TASKS = KF ? R * TK / 8 : (R / 4) * (TK / 8);
+    static constexpr int PER = (TASKS + GEMM_THREADS - 1) / GEMM_THREADS;
+    static constexpr int WIDTH = KF ? 8 : 32;
+    float v[PER][WIDTH];
+
+    static __device__ __forceinline__ void place(int task, int& r, int& kg) {
+        if constexpr (KF) {  // a warp: 8 rows x 32 columns, conflict-free stores
+            kg = ((task >> 3) & 3) | ((task >> 5) & 1) << 2;
+            r = (task & 7) | (task >> 6) << 3;
+        } else {
+            r = (task % (R / 4)) * 4;
+            kg = task / (R / 4);
         }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) *reinterpret_cast<T*>(dst + off[j]) = Cvt<T>::from(v[j]);
     }
-}
+    __device__ __forceinline__ void load(const float* __restrict__ X, int ld, bool vec, int r0, int rows, int k0, int K,
+                                         int tid) {
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int task = tid + i * GEMM_THREADS;
+            if (TASKS % GEMM_THREADS != 0 && task >= TASKS) break;
+            int r, kg;
+            place(task, r, kg);
+            const int gr = r0 + r, gk = k0 + kg * 8;
+#pragma unroll
+            for (int q = 0; q < WIDTH; q += 4) {
+                // KF: columns gk + q .. + 3 of row gr; else rows gr .. + 3 of column gk + q / 4
+                const int row = gr, col = KF ? gk + q : gk + q / 4;
+                const float* at = KF ? X + (size_t)row * ld + col : X + (size_t)col * ld + row;
+                float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (vec) {
+                    if (row < rows && col < K) f = __ldg(reinterpret_cast<const float4*>(at));
+                } else if (KF ? row < rows : col < K) {
+                    const int left = KF ? K - col : rows - row;
+                    if (left > 0) f.x = __ldg(at);
+                    if (left > 1) f.y = __ldg(at + 1);
+                    if (left > 2) f.z = __ldg(at + 2);
+                    if (left > 3) f.w = __ldg(at + 3);
+                }
+                v[i][q] = f.x;
+                v[i][q + 1] = f.y;
+                v[i][q + 2] = f.z;
+                v[i][q + 3] = f.w;
+            }
+        }
+    }
+    __device__ __forceinline__ void store(unsigned char* __restrict__ dst, int tid) const {
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int task = tid + i * GEMM_THREADS;
+            if (TASKS % GEMM_THREADS != 0 && task >= TASKS) break;
+            int r, kg;
+            place(task, r, kg);
+#pragma unroll
+            for (int j = 0; j < WIDTH / 8; ++j) {
+                T h[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) h[e] = Cvt<T>::from(KF ? v[i][e] : v[i][e * 4 + j]);
+                uint4 u;
+                memcpy(&u, h, 16);
+                *reinterpret_cast<uint4*>(dst + core_offset(r + j, kg * 8)) = u;
+            }
+        }
+    }
+};
 
 #define TMEM_LD32(taddr, r)                                                                                       \
     asm volatile(                                                                                                 \
@@ -153,21 +211,25 @@ __device__ __forceinline__ void stage_tile(unsigned char* __restrict__ dst, cons
           "=r"(r[30]), "=r"(r[31])                                                                              \
         : "r"(taddr))
 
-// C = A B with the epilogue for ensemble member blockIdx.z.  The accumulator of the
-// 128 x 64 tile lives in 64 columns of tensor memory (row m in lane m); thread 0
-// issues the MMAs of a chunk while all threads stage the next one.
-template <class T>
-__global__ void __launch_bounds__(GEMM_THREADS) gemm_kernel(GemmArgs p) {
-    extern __shared__ __align__(1024) unsigned char smem[];
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 2 * STAGE);
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + 2 * STAGE + 16);
+// One TM x TN tile of C = A B at (m0, n0) with the epilogue, for ensemble member z.
+// AF, BF: k is A's / B's contiguous index.  The accumulator lives in TN columns of
+// tensor memory (row m in lane m); thread 0 issues the MMAs of a chunk while all
+// threads load and stage the next ones.
+template <class T, int TN, bool AF, bool BF>
+__device__ __forceinline__ void gemm_tile(const GemmArgs& p, int m0, int n0, long long z, unsigned char* smem) {
+    constexpr int BASE = GEMM_SMEM<TN> - 64;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + BASE);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + BASE + 16);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
-    const long long z = blockIdx.z;
     const float* A = p.A + z * p.zA;
     const float* B = p.B + z * p.zB;
     float* C = p.C + z * p.zC;
+    const int lda = AF ? p.sam : p.sak, ldb = BF ? p.sbn : p.sbk;
     const uint32_t bar0 = smem_u32(&bars[0]), bar1 = smem_u32(&bars[1]);
+    Tile<T, TM, AF> ta;
+    Tile<T, TN, BF> tb;
+    ta.load(A, lda, p.vecA, m0, p.M, 0, p.K, tid);
+    tb.load(B, ldb, p.vecB, n0, p.N, 0, p.K, tid);
 
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)),
@@ -193,7 +255,7 @@ __global__ void __launch_bounds__(GEMM_THREADS) gemm_kernel(GemmArgs p) {
     bool failed = false;
     for (int c = 0; c < nk; ++c) {
         const int b = c & 1;
-        unsigned char* sa = smem + b * STAGE;
+        unsigned char* sa = smem + b * STAGE<TN>;
         unsigned char* sb = sa + A_TILE;
         if (c >= 2) {  // chunk c - 2 used this stage: its MMAs must have finished reading it
             const bool ok = mbar_wait_bounded(b ? bar1 : bar0, (uint32_t)(((c - 2) >> 1) & 1), p.wait_ns);
@@ -203,8 +265,12 @@ __global__ void __launch_bounds__(GEMM_THREADS) gemm_kernel(GemmArgs p) {
             }
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         }
-        stage_tile<T, TM>(sa, A, p.sam, p.sak, m0, p.M, c * TK, p.K, tid);
-        stage_tile<T, TN>(sb, B, p.sbn, p.sbk, n0, p.N, c * TK, p.K, tid);
+        ta.store(sa, tid);
+        tb.store(sb, tid);
+        if (c + 1 < nk) {
+            ta.load(A, lda, p.vecA, m0, p.M, (c + 1) * TK, p.K, tid);
+            tb.load(B, ldb, p.vecB, n0, p.N, (c + 1) * TK, p.K, tid);
+        }
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
         __syncthreads();
@@ -244,29 +310,58 @@ __global__ void __launch_bounds__(GEMM_THREADS) gemm_kernel(GemmArgs p) {
     }
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 
-    // Epilogue: warp w owns rows 32 w .. 32 w + 31 (tensor-memory lanes); 32 columns
-    // at a time go through a padded shared buffer so that a warp stores whole rows.
+    // Epilogue: warps w and w + 4 own rows 32 (w mod 4) .. + 31 (tensor-memory lanes)
+    // and take turns at blocks of 32 columns, which go through a padded shared
+    // buffer so that a warp stores whole rows.
+    const int wr = warp & 3;
     float* buf = reinterpret_cast<float*>(smem) + warp * 32 * EPI_LD;
     const float* bias = p.bias ? p.bias + z * p.zBias : nullptr;
     const float* mask = p.mask ? p.mask + z * p.zMask : nullptr;
 #pragma unroll 1
-    for (int c0 = 0; c0 < TN && n0 + c0 < p.N; c0 += 32) {
+    for (int c0 = (warp >> 2) * 32; c0 < TN && n0 + c0 < p.N; c0 += 64) {
         uint32_t r[32];
-        TMEM_LD32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0, r);
+        TMEM_LD32(tmem + ((uint32_t)(wr * 32) << 16) + (uint32_t)c0, r);
         asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
-        for (int j = 0; j < 32; ++j) buf[lane * EPI_LD + j] = __uint_as_float(r[j]);
+        for (int j = 0; j < 32; j += 4)
+            *reinterpret_cast<float4*>(buf + lane * EPI_LD + j) =
+                make_float4(__uint_as_float(r[j]), __uint_as_float(r[j + 1]), __uint_as_float(r[j + 2]),
+                            __uint_as_float(r[j + 3]));
         __syncwarp();
-        const int n = n0 + c0 + lane;
-        const float bn = (n < p.N && (p.epi == EPI_BIAS || p.epi == EPI_BIAS_RELU)) ? bias[n] : 0.f;
+        const bool with_bias = p.epi == EPI_BIAS || p.epi == EPI_BIAS_RELU;
+        if (p.vecC) {  // eight lanes a row, four rows at a time
+            const int n = n0 + c0 + (lane & 7) * 4;
+            if (n < p.N) {
+                float4 bn = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (with_bias) bn = make_float4(bias[n], bias[n + 1], bias[n + 2], bias[n + 3]);
+#pragma unroll
+                for (int rr = 0; rr < 32; rr += 4) {
+                    const int row = rr + (lane >> 3), m = m0 + wr * 32 + row;
+                    if (m >= p.M) continue;
+                    float4 v = *reinterpret_cast<const float4*>(buf + row * EPI_LD + (lane & 7) * 4);
+                    v = make_float4(v.x + bn.x, v.y + bn.y, v.z + bn.z, v.w + bn.w);
+                    if (p.epi == EPI_BIAS_RELU)
+                        v = make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f));
+                    if (p.epi == EPI_MASK) {
+                        const float4 k = __ldg(reinterpret_cast<const float4*>(mask + (size_t)m * p.ldm + n));
+                        v = make_float4(k.x > 0.f ? v.x : 0.f, k.y > 0.f ? v.y : 0.f, k.z > 0.f ? v.z : 0.f,
+                                        k.w > 0.f ? v.w : 0.f);
+                    }
+                    *reinterpret_cast<float4*>(C + (size_t)m * p.ldc + n) = v;
+                }
+            }
+        } else {
+            const int n = n0 + c0 + lane;
+            const float bn = (n < p.N && with_bias) ? bias[n] : 0.f;
 #pragma unroll 4
-        for (int rr = 0; rr < 32; ++rr) {
-            const int m = m0 + warp * 32 + rr;
-            if (m >= p.M || n >= p.N) continue;
-            float v = buf[rr * EPI_LD + lane] + bn;
-            if (p.epi == EPI_BIAS_RELU) v = fmaxf(v, 0.f);
-            if (p.epi == EPI_MASK && !(mask[(size_t)m * p.ldm + n] > 0.f)) v = 0.f;
-            C[(size_t)m * p.ldc + n] = v;
+            for (int rr = 0; rr < 32; ++rr) {
+                const int m = m0 + wr * 32 + rr;
+                if (m >= p.M || n >= p.N) continue;
+                float v = buf[rr * EPI_LD + lane] + bn;
+                if (p.epi == EPI_BIAS_RELU) v = fmaxf(v, 0.f);
+                if (p.epi == EPI_MASK && !(mask[(size_t)m * p.ldm + n] > 0.f)) v = 0.f;
+                C[(size_t)m * p.ldc + n] = v;
+            }
         }
         __syncwarp();
     }
@@ -274,6 +369,56 @@ __global__ void __launch_bounds__(GEMM_THREADS) gemm_kernel(GemmArgs p) {
     __syncthreads();
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(TN) : "memory");
+}
+
+// A layer's forward pass, member blockIdx.z: C = A B with both operands K-major.
+template <class T, int TN>
+__global__ void __launch_bounds__(GEMM_THREADS) gemm_kernel(GemmArgs p) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    gemm_tile<T, TN, true, true>(p, blockIdx.y * TM, blockIdx.x * TN, blockIdx.z, smem);
+}
+
+// db[o] = sum_b dZ[b * out + o], member z, in row order; the loads of BIAS_AHEAD
+// rows are in flight at a time (one by one, 256 rows took 10 us).
+constexpr int BIAS_AHEAD = 32, BIAS_COLS = 32;
+__device__ __forceinline__ void bias_grad(const float* __restrict__ dZ, float* __restrict__ db, int rows, int out,
+                                          int o) {
+    if (o >= out) return;
+    float s = 0.f;
+    for (int b0 = 0; b0 < rows; b0 += BIAS_AHEAD) {
+        float v[BIAS_AHEAD];
+#pragma unroll
+        for (int j = 0; j < BIAS_AHEAD; ++j) v[j] = b0 + j < rows ? __ldg(dZ + (size_t)(b0 + j) * out + o) : 0.f;
+#pragma unroll
+        for (int j = 0; j < BIAS_AHEAD; ++j)
+            if (b0 + j < rows) s += v[j];
+    }
+    db[o] = s;
+}
+
+// A layer's backward pass in one launch, member blockIdx.y: blocks below nw compute
+// tiles of dW = dZ^T H, the next nh tiles of dH = dZ W (masked), the rest bias
+// gradients.  All three only read dZ, and none alone fills the GPU.
+template <class T>
+__global__ void __launch_bounds__(GEMM_THREADS) backward_kernel(GemmArgs w, GemmArgs h, int nw, int nh, float* db,
+                                                               long long zB) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    const long long z = blockIdx.y;
+    int i = blockIdx.x;
+    if (i < nw) {
+        const int nx = (w.N + TN_SMALL - 1) / TN_SMALL;
+        gemm_tile<T, TN_SMALL, false, false>(w, i / nx * TM, i % nx * TN_SMALL, z, smem);
+        return;
+    }
+    i -= nw;
+    if (i < nh) {
+        const int nx = (h.N + TN_SMALL - 1) / TN_SMALL;
+        gemm_tile<T, TN_SMALL, true, false>(h, i / nx * TM, i % nx * TN_SMALL, z, smem);
+        return;
+    }
+    i -= nh;
+    if (threadIdx.x < BIAS_COLS)  // dZ is the weight gradient's A, K x M
+        bias_grad(w.A + z * w.zA, db + z * zB, w.K, w.M, i * BIAS_COLS + threadIdx.x);
 }
 
 // dY = loss_scale * 2 (Y - T) / (rows * cols); loss partial sums per block, for
@@ -306,27 +451,16 @@ __global__ void mse_grad_kernel(const float* __restrict__ Y, const float* __rest
     }
 }
 
-// db[o] = sum_b dZ[b * out + o], member blockIdx.y
-__global__ void bias_grad_kernel(const float* __restrict__ dZ, float* __restrict__ db, int rows, int out,
-                                 long long zZ, long long zB) {
-    const int o = blockIdx.x * blockDim.x + threadIdx.x;
-    if (o >= out) return;
-    dZ += blockIdx.y * zZ;
-    float s = 0.f;
-    for (int b = 0; b < rows; ++b) s += dZ[(size_t)b * out + o];
-    db[blockIdx.y * zB + o] = s;
-}
-
 // Bias corrections 1 - beta^t of each member (members keep their own step counts).
 struct AdamCorrections {
     float c1[64], c2[64];
 };
 
-// Adam on the flat parameters of member blockIdx.y (n per member, contiguous)
+// Adam on the flat parameters of member blockIdx.y (n per member, `stride` apart)
 __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, int n, float lr, float b1, float b2, float eps, AdamCorrections cc,
+                            float* __restrict__ v, int n, int stride, float lr, float b1, float b2, float eps, AdamCorrections cc,
                             float inv_scale) {
-    const size_t off = (size_t)blockIdx.y * n;
+    const size_t off = (size_t)blockIdx.y * stride;
     const float c1 = cc.c1[blockIdx.y], c2 = cc.c2[blockIdx.y];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const size_t j = off + i;
@@ -339,11 +473,15 @@ __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, 
     }
 }
 
-// dst (member blockIdx.y, rows x cols) = src rows idx[r]; member strides zIdx, zDst
-__global__ void gather_rows_kernel(const float* __restrict__ src, const int* __restrict__ idx, float* __restrict__ dst,
-                                   int rows, int cols, long long zIdx, long long zDst) {
+// A batch's rows of member blockIdx.y: xb = X rows idx[r] (blockIdx.z = 0), tb = T
+// rows (1); member strides zIdx, zX, zT
+__global__ void gather_rows_kernel(const float* __restrict__ X, const float* __restrict__ T,
+                                   const int* __restrict__ idx, float* __restrict__ xb, float* __restrict__ tb,
+                                   int rows, int nx, int nt, long long zIdx, long long zX, long long zT) {
     idx += blockIdx.y * zIdx;
-    dst += blockIdx.y * zDst;
+    const float* src = blockIdx.z ? T : X;
+    float* dst = blockIdx.z ? tb + blockIdx.y * zT : xb + blockIdx.y * zX;
+    const int cols = blockIdx.z ? nt : nx;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < rows * cols; i += gridDim.x * blockDim.x) {
         const int r = i / cols, c = i % cols;
         dst[i] = src[(size_t)idx[r] * cols + c];
@@ -388,9 +526,10 @@ struct lbm_surrogate {
     std::vector<size_t> w_off;  // offsets of W_l and b_l in a member's flat parameter block
     std::vector<size_t> b_off;
     size_t n_params;
-    float* params;  // [members][n_params]
-    float* grads;   // [members][n_params]
-    float* adam_m;  // [members][n_params]
+    size_t stride;  // n_params rounded up to a multiple of 4: every member's block may be read as float4
+    float* params;  // [members][stride]
+    float* grads;   // [members][stride]
+    float* adam_m;  // [members][stride]
     float* adam_v;
     int adam_t[64];
     float* acts;     // [layer input 0..L][members][cap_rows][width]
@@ -420,8 +559,10 @@ size_t act_width(const lbm_surrogate* s) {
     return w;
 }
 
-// elements between two members' buffers of one layer
-long long member_stride(const lbm_surrogate* s) { return (long long)s->cap_rows * (long long)act_width(s); }
+// elements between two members' buffers of one layer (a multiple of 4)
+long long member_stride(const lbm_surrogate* s) {
+    return ((long long)s->cap_rows * (long long)act_width(s) + 3) / 4 * 4;
+}
 
 // activation buffer of layer input l (l = 0: network input, L: output) of member z
 float* act(lbm_surrogate* s, int l, int z) {
@@ -436,7 +577,7 @@ int ensure_rows(lbm_surrogate* s, int rows) {
     cudaFree(s->dbuf[1]);
     s->acts = s->dbuf[0] = s->dbuf[1] = nullptr;
     s->cap_rows = 0;
-    const size_t per = (size_t)rows * act_width(s) * s->cfg.n_members;
+    const size_t per = ((size_t)rows * act_width(s) + 3) / 4 * 4 * s->cfg.n_members;
     SUR_CUDA(cudaMalloc(&s->acts, sizeof(float) * s->sizes.size() * per));
     SUR_CUDA(cudaMalloc(&s->dbuf[0], sizeof(float) * per));
     SUR_CUDA(cudaMalloc(&s->dbuf[1], sizeof(float) * per));
@@ -451,21 +592,53 @@ int predict_chunk(const lbm_surrogate* s) {
     return (int)std::max(128.0, std::min(16384.0, std::floor(512.0 * 1024 * 1024 / per_row)));
 }
 
-cudaError_t gemm(const lbm_surrogate* s, GemmArgs a, int members) {
-    if (a.M < 1 || a.N < 1 || a.K < 1 || members < 1) return cudaErrorInvalidValue;
+bool by4(const void* p, long long a, long long b, long long c) {
+    return (reinterpret_cast<uintptr_t>(p) & 15) == 0 && a % 4 == 0 && b % 4 == 0 && c % 4 == 0;
+}
+
+// Completes the arguments of a GEMM: the failure flag, and which of its arrays may
+// be read or written as float4 (base, row stride, extent of the contiguous index,
+// member stride).
+void finish_args(const lbm_surrogate* s, GemmArgs& a) {
     a.err = s->d_err;
     a.wait_ns = GEMM_WAIT_NS;
     a.skip_mma = 0;
-    dim3 grid((a.N + TN - 1) / TN, (a.M + TM - 1) / TM, members);
-    if (s->cfg.half) gemm_kernel<__half><<<grid, GEMM_THREADS, GEMM_SMEM, s->stream>>>(a);
-    else gemm_kernel<__nv_bfloat16><<<grid, GEMM_THREADS, GEMM_SMEM, s->stream>>>(a);
+    a.vecA = a.sak == 1 ? by4(a.A, a.sam, a.K, a.zA) : by4(a.A, a.sak, a.M, a.zA);
+    a.vecB = a.sbk == 1 ? by4(a.B, a.sbn, a.K, a.zB) : by4(a.B, a.sbk, a.N, a.zB);
+    a.vecC = by4(a.C, a.ldc, a.N, a.zC) && (!a.mask || by4(a.mask, a.ldm, a.N, a.zMask));
+}
+
+template <class T>
+cudaError_t launch_forward_gemm(const GemmArgs& a, int members, cudaStream_t st) {
+    const int my = (a.M + TM - 1) / TM;
+    // whole-width tiles once they fill the GPU by themselves (a hidden layer of 5
+    // members: from about 4000 rows on)
+    if (a.N > TN_SMALL && (long long)my * ((a.N + TN_LARGE - 1) / TN_LARGE) * members >= device_sm_count())
+        gemm_kernel<T, TN_LARGE><<<dim3((a.N + TN_LARGE - 1) / TN_LARGE, my, members), GEMM_THREADS,
+                                   GEMM_SMEM<TN_LARGE>, st>>>(a);
+    else
+        gemm_kernel<T, TN_SMALL><<<dim3((a.N + TN_SMALL - 1) / TN_SMALL, my, members), GEMM_THREADS,
+                                   GEMM_SMEM<TN_SMALL>, st>>>(a);
     return cudaGetLastError();
+}
+
+template <class T>
+cudaError_t set_gemm_smem() {
+    cudaError_t e = cudaFuncSetAttribute(gemm_kernel<T, TN_SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         GEMM_SMEM<TN_SMALL>);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(gemm_kernel<T, TN_LARGE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 GEMM_SMEM<TN_LARGE>);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(backward_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 GEMM_SMEM<TN_SMALL>);
+    return e;
 }
 
 // forward of members z0 .. z0 + nz - 1 on rows already in act(s, 0, z); with
 // shared_input every member reads the input of member z0
 int forward(lbm_surrogate* s, int z0, int nz, int rows, bool shared_input) {
-    const float* P = s->params + (size_t)z0 * s->n_params;
+    const float* P = s->params + (size_t)z0 * s->stride;
     const int L = (int)s->sizes.size() - 1;
     const long long ms = member_stride(s);
     for (int l = 0; l < L; ++l) {
@@ -475,7 +648,7 @@ int forward(lbm_surrogate* s, int z0, int nz, int rows, bool shared_input) {
         a.sam = s->sizes[l];
         a.sak = 1;
         a.B = P + s->w_off[l];  // B(k, n) = W[n][k]
-        a.zB = (long long)s->n_params;
+        a.zB = (long long)s->stride;
         a.sbk = 1;
         a.sbn = s->sizes[l];
         a.C = act(s, l + 1, z0);
@@ -485,9 +658,12 @@ int forward(lbm_surrogate* s, int z0, int nz, int rows, bool shared_input) {
         a.N = s->sizes[l + 1];
         a.K = s->sizes[l];
         a.bias = P + s->b_off[l];
-        a.zBias = (long long)s->n_params;
+        a.zBias = (long long)s->stride;
         a.epi = l < L - 1 ? EPI_BIAS_RELU : EPI_BIAS;
-        SUR_CUDA(gemm(s, a, nz));
+        if (a.M < 1 || nz < 1) SUR_CUDA(cudaErrorInvalidValue);
+        finish_args(s, a);
+        SUR_CUDA(s->cfg.half ? launch_forward_gemm<__half>(a, nz, s->stream)
+                             : launch_forward_gemm<__nv_bfloat16>(a, nz, s->stream));
     }
     return LBM_OK;
 }
@@ -497,9 +673,9 @@ int forward(lbm_surrogate* s, int z0, int nz, int rows, bool shared_input) {
 // added to loss_acc[z * zL] (device)
 int backward(lbm_surrogate* s, int z0, int nz, int rows, const float* T, long long zT, double* loss_acc,
              long long zL) {
-    const float* P = s->params + (size_t)z0 * s->n_params;
-    float* G = s->grads + (size_t)z0 * s->n_params;
-    const long long np = (long long)s->n_params, ms = member_stride(s);
+    const float* P = s->params + (size_t)z0 * s->stride;
+    float* G = s->grads + (size_t)z0 * s->stride;
+    const long long np = (long long)s->stride, ms = member_stride(s);
     const int L = (int)s->sizes.size() - 1;
     const int nout = s->sizes[L];
     float* dz = dbuf(s, 0, z0);
@@ -526,11 +702,10 @@ int backward(lbm_surrogate* s, int z0, int nz, int rows, const float* T, long lo
         g.N = in;
         g.K = rows;
         g.epi = EPI_NONE;
-        SUR_CUDA(gemm(s, g, nz));
-        bias_grad_kernel<<<dim3((out + 127) / 128, nz), 128, 0, s->stream>>>(dz, G + s->b_off[l], rows, out, ms, np);
-        SUR_CUDA(cudaGetLastError());
-        if (l > 0) {
-            GemmArgs d{};  // dH = dZ W, masked by ReLU'(z_{l-1}) = [h_l > 0]
+        finish_args(s, g);
+        auto tiles = [](const GemmArgs& a) { return ((a.M + TM - 1) / TM) * ((a.N + TN_SMALL - 1) / TN_SMALL); };
+        GemmArgs d{};
+        if (l > 0) {  // dH = dZ W, masked by ReLU'(z_{l-1}) = [h_l > 0]
             d.A = dz;
             d.zA = ms;
             d.sam = out;
@@ -549,9 +724,17 @@ int backward(lbm_surrogate* s, int z0, int nz, int rows, const float* T, long lo
             d.zMask = ms;
             d.ldm = in;
             d.epi = EPI_MASK;
-            SUR_CUDA(gemm(s, d, nz));
-            std::swap(dz, dh);
+            finish_args(s, d);
         }
+        const int nw = tiles(g), nh = l > 0 ? tiles(d) : 0, nb = (out + BIAS_COLS - 1) / BIAS_COLS;
+        if (s->cfg.half)
+            backward_kernel<__half><<<dim3(nw + nh + nb, nz), GEMM_THREADS, GEMM_SMEM<TN_SMALL>, s->stream>>>(
+                g, d, nw, nh, G + s->b_off[l], np);
+        else
+            backward_kernel<__nv_bfloat16><<<dim3(nw + nh + nb, nz), GEMM_THREADS, GEMM_SMEM<TN_SMALL>, s->stream>>>(
+                g, d, nw, nh, G + s->b_off[l], np);
+        SUR_CUDA(cudaGetLastError());
+        if (l > 0) std::swap(dz, dh);
     }
     return LBM_OK;
 }
@@ -565,9 +748,9 @@ int adam(lbm_surrogate* s, int z0, int nz, float lr) {
         cc.c2[z] = 1.f - std::pow(b2, (float)t);
     }
     const int n = (int)s->n_params;
-    const size_t off = (size_t)z0 * s->n_params;
+    const size_t off = (size_t)z0 * s->stride;
     adam_kernel<<<dim3(std::min(1024, (n + 255) / 256), nz), 256, 0, s->stream>>>(
-        s->params + off, s->grads + off, s->adam_m + off, s->adam_v + off, n, lr, b1, b2, eps, cc, 1.0f / LOSS_SCALE);
+        s->params + off, s->grads + off, s->adam_m + off, s->adam_v + off, n, (int)s->stride, lr, b1, b2, eps, cc, 1.0f / LOSS_SCALE);
     SUR_CUDA(cudaGetLastError());
     return LBM_OK;
 }
@@ -609,8 +792,9 @@ int lbm_surrogate_create(const lbm_surrogate_config* cfg, void* stream, lbm_surr
         off += (size_t)s->sizes[l + 1];
     }
     s->n_params = off;
+    s->stride = (off + 3) / 4 * 4;
     // seeded He-normal weights, zero biases, per member
-    std::vector<float> init(s->n_params * cfg->n_members, 0.f);
+    std::vector<float> init(s->stride * cfg->n_members, 0.f);
     for (int m = 0; m < cfg->n_members; ++m) {
         uint64_t st = cfg->seed * 0x100000001B3ull + (uint64_t)m * 0x9E3779B97F4A7C15ull + 1;
         for (size_t l = 0; l + 1 < s->sizes.size(); ++l) {
@@ -618,13 +802,13 @@ int lbm_surrogate_create(const lbm_surrogate_config* cfg, void* stream, lbm_surr
             const size_t nw = (size_t)s->sizes[l] * s->sizes[l + 1];
             for (size_t i = 0; i < nw; ++i) {
                 const double u1 = uniform01(st), u2 = uniform01(st);
-                init[m * s->n_params + s->w_off[l] + i] =
+                init[m * s->stride + s->w_off[l] + i] =
                     (float)(sd * std::sqrt(-2.0 * std::log(u1)) * std::cos(6.283185307179586 * u2));
             }
         }
     }
     auto bail = [&](int rc) { lbm_surrogate_destroy(s); return rc; };
-    const size_t pb = sizeof(float) * s->n_params * cfg->n_members;
+    const size_t pb = sizeof(float) * s->stride * cfg->n_members;
     cudaError_t e;
     if ((e = cudaMalloc(&s->params, pb)) != cudaSuccess) return bail(sur_fail(e, "cudaMalloc"));
     if ((e = cudaMalloc(&s->adam_m, pb)) != cudaSuccess) return bail(sur_fail(e, "cudaMalloc"));
@@ -633,10 +817,7 @@ int lbm_surrogate_create(const lbm_surrogate_config* cfg, void* stream, lbm_surr
     if ((e = cudaMalloc(&s->d_loss, sizeof(double))) != cudaSuccess) return bail(sur_fail(e, "cudaMalloc"));
     if ((e = cudaMalloc(&s->d_err, sizeof(int))) != cudaSuccess) return bail(sur_fail(e, "cudaMalloc"));
     if ((e = cudaMemsetAsync(s->d_err, 0, sizeof(int), s->stream)) != cudaSuccess) return bail(sur_fail(e, "memset"));
-    if ((e = cudaFuncSetAttribute(gemm_kernel<__half>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM)) !=
-            cudaSuccess ||
-        (e = cudaFuncSetAttribute(gemm_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  GEMM_SMEM)) != cudaSuccess)
+    if ((e = set_gemm_smem<__half>()) != cudaSuccess || (e = set_gemm_smem<__nv_bfloat16>()) != cudaSuccess)
         return bail(sur_fail(e, "cudaFuncSetAttribute"));
     if ((e = cudaMemcpyAsync(s->params, init.data(), pb, cudaMemcpyHostToDevice, s->stream)) != cudaSuccess)
         return bail(sur_fail(e, "cudaMemcpyAsync"));
@@ -651,7 +832,7 @@ int lbm_surrogate_num_params(const lbm_surrogate* s) { return s ? (int)s->n_para
 
 int lbm_surrogate_get_params(lbm_surrogate* s, int member, float* out) {
     if (!s || !out || member < 0 || member >= s->cfg.n_members) { set_error("bad argument"); return LBM_ERR_ARG; }
-    SUR_CUDA(cudaMemcpyAsync(out, s->params + (size_t)member * s->n_params, sizeof(float) * s->n_params,
+    SUR_CUDA(cudaMemcpyAsync(out, s->params + (size_t)member * s->stride, sizeof(float) * s->n_params,
                              cudaMemcpyDeviceToHost, s->stream));
     SUR_CUDA(cudaStreamSynchronize(s->stream));
     return LBM_OK;
@@ -659,12 +840,12 @@ int lbm_surrogate_get_params(lbm_surrogate* s, int member, float* out) {
 
 int lbm_surrogate_set_params(lbm_surrogate* s, int member, const float* in) {
     if (!s || !in || member < 0 || member >= s->cfg.n_members) { set_error("bad argument"); return LBM_ERR_ARG; }
-    SUR_CUDA(cudaMemcpyAsync(s->params + (size_t)member * s->n_params, in, sizeof(float) * s->n_params,
+    SUR_CUDA(cudaMemcpyAsync(s->params + (size_t)member * s->stride, in, sizeof(float) * s->n_params,
                              cudaMemcpyHostToDevice, s->stream));
     SUR_CUDA(cudaStreamSynchronize(s->stream));
     s->adam_t[member] = 0;
-    SUR_CUDA(cudaMemsetAsync(s->adam_m + (size_t)member * s->n_params, 0, sizeof(float) * s->n_params, s->stream));
-    SUR_CUDA(cudaMemsetAsync(s->adam_v + (size_t)member * s->n_params, 0, sizeof(float) * s->n_params, s->stream));
+    SUR_CUDA(cudaMemsetAsync(s->adam_m + (size_t)member * s->stride, 0, sizeof(float) * s->n_params, s->stream));
+    SUR_CUDA(cudaMemsetAsync(s->adam_v + (size_t)member * s->stride, 0, sizeof(float) * s->n_params, s->stream));
     return LBM_OK;
 }
 
@@ -701,7 +882,7 @@ int lbm_surrogate_gradients(lbm_surrogate* s, int member, const float* X, const 
     if (!rc) rc = backward(s, member, 1, n, dT, 0, s->d_loss, 0);
     cudaFreeAsync(dT, s->stream);
     if (rc) return rc;
-    SUR_CUDA(cudaMemcpyAsync(grads, s->grads + (size_t)member * s->n_params, sizeof(float) * s->n_params,
+    SUR_CUDA(cudaMemcpyAsync(grads, s->grads + (size_t)member * s->stride, sizeof(float) * s->n_params,
                              cudaMemcpyDeviceToHost, s->stream));
     double l = 0;
     SUR_CUDA(cudaMemcpyAsync(&l, s->d_loss, sizeof(double), cudaMemcpyDeviceToHost, s->stream));
@@ -760,10 +941,9 @@ int lbm_surrogate_train(lbm_surrogate* s, const float* X, const float* T, int n,
     for (int ep = 0; ep < epochs; ++ep) {
         for (int b0 = 0; b0 + batch <= n; b0 += batch) {
             const int* idx = dIdx + (size_t)ep * n + b0;
-            gather_rows_kernel<<<dim3(std::min(1024, (batch * nin + 255) / 256), M), 256, 0, s->stream>>>(
-                dX, idx, act(s, 0, 0), batch, nin, (long long)E * n, ms);
-            gather_rows_kernel<<<dim3(std::min(1024, (batch * nout + 255) / 256), M), 256, 0, s->stream>>>(
-                dT, idx, dTb, batch, nout, (long long)E * n, (long long)batch * nout);
+            gather_rows_kernel<<<dim3(std::min(1024, (batch * std::max(nin, nout) + 255) / 256), M, 2), 256, 0,
+                                 s->stream>>>(dX, dT, idx, act(s, 0, 0), dTb, batch, nin, nout, (long long)E * n, ms,
+                                              (long long)batch * nout);
             TR_CUDA(cudaGetLastError());
             int rc = forward(s, 0, M, batch, false);
             if (!rc) rc = backward(s, 0, M, batch, dTb, (long long)batch * nout, dLoss + ep, E);
@@ -833,8 +1013,7 @@ int lbm_surrogate_selftest_wait(int limit_us, int* gave_up) {
     cudaError_t e = cudaMalloc(&d_flag, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(buf, 0, sizeof(float) * 4);
     if (e == cudaSuccess) e = cudaMemset(d_flag, 0, sizeof(int));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(gemm_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM);
+    if (e == cudaSuccess) e = set_gemm_smem<__nv_bfloat16>();
     if (e == cudaSuccess) {
         GemmArgs a{};
         a.A = buf;
@@ -846,7 +1025,7 @@ int lbm_surrogate_selftest_wait(int limit_us, int* gave_up) {
         a.err = d_flag;
         a.wait_ns = 1000ull * (unsigned long long)limit_us;
         a.skip_mma = 1;  // no MMA and no commit: the completion barrier never completes
-        gemm_kernel<__nv_bfloat16><<<1, GEMM_THREADS, GEMM_SMEM>>>(a);
+        gemm_kernel<__nv_bfloat16, TN_SMALL><<<1, GEMM_THREADS, (GEMM_SMEM<TN_SMALL>)>>>(a);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
