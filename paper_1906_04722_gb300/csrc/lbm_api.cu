@@ -1,4 +1,5 @@
 // lbm_api.cu -- the extern "C" entry points declared in include/lbm.h.
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
@@ -279,6 +280,7 @@ void free_domain(lbm_domain* d) {
     cudaFree(d->d_nbr_nw);
     cudaFree(d->d_adh);
     cudaFree(d->d_rho);
+    cudaFree(d->d_convert);
     cudaFree(d->d_partials);
     cudaFree(d->d_result);
     cudaFree(d->d_bc);
@@ -293,7 +295,9 @@ void free_domain(lbm_domain* d) {
     delete d;
 }
 
-// Bounded wait for the domain's queued work: polls an event for up to 60 s.
+// Bounded wait for the domain's queued work: polls an event for up to 60 s, without
+// sleeping for the first milliseconds (a throat's read-out takes tens of
+// microseconds, a sleep of 50 us about 110).
 int wait_domain(lbm_domain* d) {
     // a TMA step kernel whose bounded wait for its loads ran out leaves a flag:
     // read it on the domain's stream, behind the work being waited for
@@ -319,11 +323,13 @@ int wait_domain(lbm_domain* d) {
             set_error(std::string("device work failed: ") + cudaGetErrorString(e));
             return LBM_ERR_CUDA;
         }
-        if (std::chrono::steady_clock::now() - t0 > std::chrono::seconds(60)) {
+        const auto waited = std::chrono::steady_clock::now() - t0;
+        if (waited > std::chrono::seconds(60)) {
             set_error("device work did not finish within 60 s");
             return LBM_ERR_TIMEOUT;
         }
-        std::this_thread::sleep_for(std::chrono::microseconds(50));
+        if (waited < std::chrono::milliseconds(5)) std::this_thread::yield();
+        else std::this_thread::sleep_for(std::chrono::microseconds(50));
     }
 }
 
@@ -336,6 +342,18 @@ __global__ void rest_density_kernel(const uint8_t* __restrict__ mask, float* __r
         rho[c] = inlet ? rho_minor : rho_major;
         rho[N + c] = inlet ? rho_major : rho_minor;
     }
+}
+
+// Densities between the host's doubles and the device's floats, converted on the
+// device piece by piece (a host loop over the 192^3 sample's 14 M values took 8 ms).
+constexpr long long CONVERT_PIECE = 4LL << 20;  // doubles
+__global__ void to_float_kernel(const double* __restrict__ in, float* __restrict__ out, long long n) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        out[i] = (float)in[i];
+}
+__global__ void to_double_kernel(const float* __restrict__ in, double* __restrict__ out, long long n) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        out[i] = (double)in[i];
 }
 
 // Build the stored populations from the densities in d->d_rho.
@@ -356,11 +374,82 @@ int init_from_densities(lbm_domain* d) {
 // Upload rest-equilibrium densities (host doubles, 2 x N) and build the stored
 // populations from them.
 int upload_densities(lbm_domain* d, const double* rho) {
-    const long long N = d->N;
-    std::vector<float> tmp((size_t)(2 * N));
-    for (long long i = 0; i < 2 * N; ++i) tmp[(size_t)i] = (float)rho[i];
-    LBM_CUDA(cudaMemcpyAsync(d->d_rho, tmp.data(), sizeof(float) * 2 * N, cudaMemcpyHostToDevice, d->stream));
+    for (long long i = 0; i < 2 * d->N; i += CONVERT_PIECE) {
+        const long long n = std::min(CONVERT_PIECE, 2 * d->N - i);
+        LBM_CUDA(cudaMemcpyAsync(d->d_convert, rho + i, sizeof(double) * n, cudaMemcpyHostToDevice, d->stream));
+        to_float_kernel<<<1216, 256, 0, d->stream>>>(d->d_convert, d->d_rho + i, n);
+        LBM_CUDA(cudaGetLastError());
+    }
     return init_from_densities(d);
+}
+
+// Queue the measurement of the current state, its sums going to h_result; after a
+// wait, read_measurement gives the observables.
+int queue_measure(lbm_domain* d) {
+    if (d->params.precision == 0 && d->layout == 1) {
+        LBM_CUDA(launch_measure_push(d->f[d->cur], d->d_nbr, d->geom, d->params.G, d->d_partials, d->meas_blocks,
+                                     d->d_result, d->stream));
+    } else if (d->params.precision == 0) {
+        LBM_CUDA(launch_measure(d->f[d->cur], d->d_nbr, d->d_nbr_nw, d->geom, d->params.G, d->d_partials,
+                                d->meas_blocks, d->d_result, d->stream));
+    }
+    else {
+        LBM_CUDA(launch_measure16(d->params.precision, reinterpret_cast<const uint32_t*>(d->f[d->cur]), d->R[d->cur],
+                                  d->d_nbr, d->d_nbr_nw, d->geom, d->layout == 1, d->params.G, d->d_partials,
+                                  d->meas_blocks, d->d_result, d->stream));
+    }
+    LBM_CUDA(cudaMemcpyAsync(d->h_result, d->d_result, sizeof(double) * NMEAS, cudaMemcpyDeviceToHost, d->stream));
+    return LBM_OK;
+}
+
+int read_measurement(lbm_domain* d, lbm_measurement* out) {
+    const double* r = d->h_result;
+    std::memset(out, 0, sizeof(*out));
+    out->mass[0] = r[MS_MASS_W];
+    out->mass[1] = r[MS_MASS_NW];
+    out->n_fluid = (long long)r[MS_N_FLUID];
+    out->n_w = (long long)r[MS_N_W];
+    out->n_interface = (long long)r[MS_N_INTERFACE];
+    out->n_bulk_w = (long long)r[MS_N_BULK_W];
+    out->n_bulk_nw = (long long)r[MS_N_BULK_NW];
+    out->n_in = (long long)r[MS_N_IN];
+    out->n_out = (long long)r[MS_N_OUT];
+    out->n_nonfinite = (long long)r[MS_N_NONFINITE];
+    out->n_negative = (long long)r[MS_N_NEGATIVE];
+    out->p_w = out->n_bulk_w ? r[MS_PW] / (double)out->n_bulk_w : NAN;
+    out->p_nw = out->n_bulk_nw ? r[MS_PNW] / (double)out->n_bulk_nw : NAN;
+    out->p_c = out->p_nw - out->p_w;
+    out->p_in = out->n_in ? r[MS_PIN] / (double)out->n_in : NAN;
+    out->p_out = out->n_out ? r[MS_POUT] / (double)out->n_out : NAN;
+    out->p_c_res = out->p_in - out->p_out;
+    out->S_w = out->n_fluid ? (double)out->n_w / (double)out->n_fluid : NAN;
+    out->status_flags = (out->n_nonfinite ? 1 : 0) | (out->n_negative ? 2 : 0);
+    if (out->status_flags) {
+        set_error("non-finite or negative densities in the state");
+        return LBM_ERR_NONFINITE;
+    }
+    return LBM_OK;
+}
+
+// Queue the densities of one cell; after a wait they are at probe_result.
+const float* probe_result(const lbm_domain* d) { return reinterpret_cast<const float*>(d->h_result + NMEAS); }
+
+int queue_probe(lbm_domain* d, int x, int y, int z) {
+    if (x < 0 || y < 0 || z < 0 || x >= d->geom.nx || y >= d->geom.ny || z >= d->geom.nz) {
+        set_error("probe cell outside the box");
+        return LBM_ERR_ARG;
+    }
+    if (d->params.precision == 0 && d->layout == 1) {
+        LBM_CUDA(launch_probe_push(d->f[d->cur], d->d_nbr, d->geom, x, y, z, d->d_probe, d->stream));
+    } else if (d->params.precision == 0) {
+        LBM_CUDA(launch_probe(d->f[d->cur], d->d_nbr, d->d_nbr_nw, d->geom, x, y, z, d->d_probe, d->stream));
+    }
+    else {
+        LBM_CUDA(launch_probe16(d->params.precision, reinterpret_cast<const uint32_t*>(d->f[d->cur]), d->R[d->cur],
+                                d->d_nbr, d->d_nbr_nw, d->geom, d->layout == 1, x, y, z, d->d_probe, d->stream));
+    }
+    LBM_CUDA(cudaMemcpyAsync(d->h_result + NMEAS, d->d_probe, sizeof(float) * 2, cudaMemcpyDeviceToHost, d->stream));
+    return LBM_OK;
 }
 
 int create_common(const lbm_params* params, const uint8_t* mask_host, const int box[3], void* stream,
@@ -416,10 +505,11 @@ int create_common(const lbm_params* params, const uint8_t* mask_host, const int 
     LBM_CUDA_D(cudaMalloc(&d->d_nbr_nw, sizeof(uint32_t) * (size_t)d->N));
     LBM_CUDA_D(cudaMalloc(&d->d_adh, sizeof(uint32_t) * (size_t)d->N));
     LBM_CUDA_D(cudaMalloc(&d->d_rho, sizeof(float) * 2 * (size_t)d->N));
+    LBM_CUDA_D(cudaMalloc(&d->d_convert, sizeof(double) * (size_t)std::min(CONVERT_PIECE, 2 * d->N)));
     d->meas_blocks = measure_blocks(g);
     LBM_CUDA_D(cudaMalloc(&d->d_partials, sizeof(double) * NMEAS * (size_t)d->meas_blocks));
     LBM_CUDA_D(cudaMalloc(&d->d_result, sizeof(double) * NMEAS));
-    LBM_CUDA_D(cudaMallocHost(&d->h_result, sizeof(double) * NMEAS));
+    LBM_CUDA_D(cudaMallocHost(&d->h_result, sizeof(double) * (NMEAS + 1)));
     LBM_CUDA_D(cudaMalloc(&d->d_bc, sizeof(float) * 4));
     LBM_CUDA_D(cudaMalloc(&d->d_probe, sizeof(float) * 2));
     LBM_CUDA_D(cudaMalloc(&d->d_err, sizeof(int)));
@@ -544,23 +634,10 @@ int lbm_step(lbm_domain* d, int n_steps) {
 
 int lbm_get_density_at(lbm_domain* d, int x, int y, int z, double rho_out[2]) {
     if (!d || !rho_out) { set_error("domain or rho_out is NULL"); return LBM_ERR_ARG; }
-    if (x < 0 || y < 0 || z < 0 || x >= d->geom.nx || y >= d->geom.ny || z >= d->geom.nz) {
-        set_error("probe cell outside the box");
-        return LBM_ERR_ARG;
-    }
-    if (d->params.precision == 0 && d->layout == 1) {
-        LBM_CUDA(launch_probe_push(d->f[d->cur], d->d_nbr, d->geom, x, y, z, d->d_probe, d->stream));
-    } else if (d->params.precision == 0) {
-        LBM_CUDA(launch_probe(d->f[d->cur], d->d_nbr, d->d_nbr_nw, d->geom, x, y, z, d->d_probe, d->stream));
-    }
-    else {
-        LBM_CUDA(launch_probe16(d->params.precision, reinterpret_cast<const uint32_t*>(d->f[d->cur]), d->R[d->cur],
-                                d->d_nbr, d->d_nbr_nw, d->geom, d->layout == 1, x, y, z, d->d_probe, d->stream));
-    }
-    LBM_CUDA(cudaMemcpyAsync(d->h_result, d->d_probe, sizeof(float) * 2, cudaMemcpyDeviceToHost, d->stream));
-    int rc = wait_domain(d);
+    int rc = queue_probe(d, x, y, z);
+    if (!rc) rc = wait_domain(d);
     if (rc) return rc;
-    const float* r = reinterpret_cast<const float*>(d->h_result);
+    const float* r = probe_result(d);
     rho_out[0] = r[0];
     rho_out[1] = r[1];
     return LBM_OK;
@@ -578,12 +655,18 @@ int lbm_run_drainage(lbm_domain* d, const double* rho_in_nw, int n_incr, int n_s
         if (rc) return rc;
         rc = run_steps(d, n_steps);
         if (rc) return rc;
+        // measurement and probe behind the steps, one wait for all
         lbm_measurement m;
-        rc = lbm_measure(d, &m);
+        rc = queue_measure(d);
+        const int rp = rc ? rc : queue_probe(d, probe[0], probe[1], probe[2]);
+        if (!rc) rc = wait_domain(d);
+        if (!rc) rc = read_measurement(d, &m);
         if (rc && rc != LBM_ERR_NONFINITE) return rc;
-        double pr[2];
-        int rp = lbm_get_density_at(d, probe[0], probe[1], probe[2], pr);
-        if (rp) return rp;
+        if (rp) {
+            if (rp == LBM_ERR_ARG) set_error("probe cell outside the box");
+            return rp;
+        }
+        const double pr[2] = {probe_result(d)[0], probe_result(d)[1]};
         lbm_increment& r = rows[i];
         r.rho_in_nw = rho_in_nw[i];
         r.p_c = m.p_c;
@@ -611,47 +694,9 @@ int lbm_run_drainage(lbm_domain* d, const double* rho_in_nw, int n_incr, int n_s
 
 int lbm_measure(lbm_domain* d, lbm_measurement* out) {
     if (!d || !out) { set_error("domain or out is NULL"); return LBM_ERR_ARG; }
-    if (d->params.precision == 0 && d->layout == 1) {
-        LBM_CUDA(launch_measure_push(d->f[d->cur], d->d_nbr, d->geom, d->params.G, d->d_partials, d->meas_blocks,
-                                     d->d_result, d->stream));
-    } else if (d->params.precision == 0) {
-        LBM_CUDA(launch_measure(d->f[d->cur], d->d_nbr, d->d_nbr_nw, d->geom, d->params.G, d->d_partials,
-                                d->meas_blocks, d->d_result, d->stream));
-    }
-    else {
-        LBM_CUDA(launch_measure16(d->params.precision, reinterpret_cast<const uint32_t*>(d->f[d->cur]), d->R[d->cur],
-                                  d->d_nbr, d->d_nbr_nw, d->geom, d->layout == 1, d->params.G, d->d_partials,
-                                  d->meas_blocks, d->d_result, d->stream));
-    }
-    LBM_CUDA(cudaMemcpyAsync(d->h_result, d->d_result, sizeof(double) * NMEAS, cudaMemcpyDeviceToHost, d->stream));
-    int rc = wait_domain(d);
-    if (rc) return rc;
-    const double* r = d->h_result;
-    std::memset(out, 0, sizeof(*out));
-    out->mass[0] = r[MS_MASS_W];
-    out->mass[1] = r[MS_MASS_NW];
-    out->n_fluid = (long long)r[MS_N_FLUID];
-    out->n_w = (long long)r[MS_N_W];
-    out->n_interface = (long long)r[MS_N_INTERFACE];
-    out->n_bulk_w = (long long)r[MS_N_BULK_W];
-    out->n_bulk_nw = (long long)r[MS_N_BULK_NW];
-    out->n_in = (long long)r[MS_N_IN];
-    out->n_out = (long long)r[MS_N_OUT];
-    out->n_nonfinite = (long long)r[MS_N_NONFINITE];
-    out->n_negative = (long long)r[MS_N_NEGATIVE];
-    out->p_w = out->n_bulk_w ? r[MS_PW] / (double)out->n_bulk_w : NAN;
-    out->p_nw = out->n_bulk_nw ? r[MS_PNW] / (double)out->n_bulk_nw : NAN;
-    out->p_c = out->p_nw - out->p_w;
-    out->p_in = out->n_in ? r[MS_PIN] / (double)out->n_in : NAN;
-    out->p_out = out->n_out ? r[MS_POUT] / (double)out->n_out : NAN;
-    out->p_c_res = out->p_in - out->p_out;
-    out->S_w = out->n_fluid ? (double)out->n_w / (double)out->n_fluid : NAN;
-    out->status_flags = (out->n_nonfinite ? 1 : 0) | (out->n_negative ? 2 : 0);
-    if (out->status_flags) {
-        set_error("non-finite or negative densities in the state");
-        return LBM_ERR_NONFINITE;
-    }
-    return LBM_OK;
+    int rc = queue_measure(d);
+    if (!rc) rc = wait_domain(d);
+    return rc ? rc : read_measurement(d, out);
 }
 
 int lbm_get_density(lbm_domain* d, double* rho_out) {
@@ -667,12 +712,13 @@ int lbm_get_density(lbm_domain* d, double* rho_out) {
                                       d->R[d->cur], d->d_nbr, d->d_nbr_nw, d->geom, d->layout == 1, d->d_rho,
                                       d->stream));
         }
-        std::vector<float> tmp((size_t)(2 * d->N));
-        LBM_CUDA(cudaMemcpyAsync(tmp.data(), d->d_rho, sizeof(float) * 2 * d->N, cudaMemcpyDeviceToHost, d->stream));
-        int rc = wait_domain(d);
-        if (rc) return rc;
-        for (long long i = 0; i < 2 * d->N; ++i) rho_out[i] = tmp[(size_t)i];
-        return LBM_OK;
+        for (long long i = 0; i < 2 * d->N; i += CONVERT_PIECE) {
+            const long long n = std::min(CONVERT_PIECE, 2 * d->N - i);
+            to_double_kernel<<<1216, 256, 0, d->stream>>>(d->d_rho + i, d->d_convert, n);
+            LBM_CUDA(cudaGetLastError());
+            LBM_CUDA(cudaMemcpyAsync(rho_out + i, d->d_convert, sizeof(double) * n, cudaMemcpyDeviceToHost, d->stream));
+        }
+        return wait_domain(d);
     } catch (const std::bad_alloc&) {
         set_error("host allocation failed");
         return LBM_ERR_OOM;

@@ -238,9 +238,10 @@ struct lbm_domain {
     uint32_t* d_nbr_nw;
     uint32_t* d_adh;
     float* d_rho;
+    double* d_convert;  // a piece of the density field in doubles, for the host's copies
     double* d_partials;
     double* d_result;
-    double* h_result;  // pinned
+    double* h_result;  // pinned: the measurement's sums, then a probe cell's densities
     int meas_blocks;
     cudaStream_t stream;
     cudaEvent_t done;
