@@ -586,7 +586,11 @@ int lbm_get_tile(const lbm_domain* d, int* by, int* lz, int* lead);
  *                      lz planes per CTA z-segment (lz <= 0: the default);
  *   LBM_KERNEL_SPLIT   two launches per step: every cell's density pair into a
  *                      field, then pull + collision reading the 18 neighbour
- *                      densities from it (any box; FP32 only; lz ignored);
+ *                      densities from it (any box; FP32 only; lz ignored); with
+ *                      tau = 1 in both components on the paired push layout
+ *                      below, the second launch working from densities and
+ *                      velocities alone (the staged kernel's results bit for
+ *                      bit);
  *   LBM_KERNEL_STAGED2 the staged kernel with two threads per cell, one per
  *                      fluid component (any box; FP32 only; by 6 or 8, lead 2,
  *                      lz planes per z segment, lz <= 0: keep the current).
@@ -614,7 +618,9 @@ int lbm_get_tile(const lbm_domain* d, int* by, int* lz, int* lead);
  *                      and with nx % 4 == 0).  Its results equal the staged
  *                      16-bit kernel's bit for bit; the read-outs read
  *                      either layout.
- * New domains use LBM_KERNEL_STAGED (lbm_autotune times every kind that applies
+ * New domains use LBM_KERNEL_STAGED; as long as neither a kernel nor a shape has
+ * been chosen, an FP32 domain with tau = 1 in both components steps through the
+ * two launches of LBM_KERNEL_SPLIT, with the same bits (lbm_autotune times every kind that applies
  * on the domain).  All give the same results up to rounding (not bit for bit:
  * the TMA kernel folds omega w_k into its equilibrium constants).  LBM_ERR_ARG
  * for an unknown kind, LBM_ERR_STATE when the kernel does not apply to the

@@ -97,8 +97,21 @@ void drop_graphs(lbm_domain* d) {
         }
 }
 
+// Whether steps run as the two launches of lbm_step_pairs.cu: the two-launch kernel
+// at tau = 1, and a domain that nobody has chosen a kernel for -- the results are
+// the staged kernel's bit for bit, and on every box measured it is the faster one
+// (a step of a 32^3 throat 10.4 -> 4.2 us, 48^3 periodic 16.1 -> 7.1 us, the 192^3
+// sample 0.69 -> 0.49 ms).
+bool steps_in_pairs(const lbm_domain* d) {
+    return d->params.precision == 0 && pair_step_applicable(d->phys) &&
+           (d->tile.kind == LBM_KERNEL_SPLIT || (d->tile.kind == LBM_KERNEL_STAGED && !d->chosen));
+}
+
 // One step from buffer `cur` to buffer cur ^ 1 on stream s.
 cudaError_t launch_one(lbm_domain* d, int cur, cudaStream_t s) {
+    if (steps_in_pairs(d))
+        return launch_step_pairs(d->f[cur], d->f[cur ^ 1], d->d_rho2, d->d_nbr, d->d_nbr_nw, d->d_adh, d->geom,
+                                 d->phys, s);
     if (d->params.precision != 0 && d->tile.kind == LBM_KERNEL_PUSH)
         return launch_step16_push(d->params.precision, d->tile.push_shape, d->push16_w[cur], d->push16_r[cur],
                                   reinterpret_cast<uint32_t*>(d->f[cur ^ 1]), d->R[cur ^ 1], d->d_nbr, d->d_nbr_nw,
@@ -122,6 +135,7 @@ cudaError_t launch_one(lbm_domain* d, int cur, cudaStream_t s) {
 }
 
 cudaError_t prepare_one(lbm_domain* d) {
+    if (steps_in_pairs(d)) return cudaSuccess;
     if (d->params.precision != 0 && d->tile.kind == LBM_KERNEL_PUSH)
         return prepare_step16_push(d->params.precision, d->tile.push_shape);
     if (d->params.precision == 0 && d->tile.kind == LBM_KERNEL_PUSH) return prepare_step_push(d->tile.push_shape);
@@ -131,10 +145,10 @@ cudaError_t prepare_one(lbm_domain* d) {
     return d->params.precision == 0 ? prepare_step(d->tile) : prepare_step16(d->params.precision, d->tile);
 }
 
-// The layout the current kernel kind steps on: the push kernels keep the state
-// in the push layout (FP32: paired; 16-bit: the pull words, each at its reader),
-// every other kernel in the pull layout.
-int wanted_layout(const lbm_domain* d) { return d->tile.kind == LBM_KERNEL_PUSH ? 1 : 0; }
+// The layout the current kernel kind steps on: the push kernels and the two-launch
+// kernel at tau = 1 keep the state in the push layout (FP32: paired; 16-bit: the
+// pull words, each at its reader), every other kernel in the pull layout.
+int wanted_layout(const lbm_domain* d) { return d->tile.kind == LBM_KERNEL_PUSH || steps_in_pairs(d) ? 1 : 0; }
 
 // Converts the state into the given layout (into the other buffer, which then
 // becomes the current one).  The step counter is unchanged.
@@ -778,6 +792,7 @@ int lbm_set_tile(lbm_domain* d, int by, int lz, int lead) {
     d->tile.lz = lz > d->geom.nz ? d->geom.nz : lz;
     d->tile.lead = lead;
     d->tile.kind = LBM_KERNEL_STAGED;
+    d->chosen = true;
     drop_graphs(d);  // captured with the old shape
     return LBM_OK;
 }
@@ -798,6 +813,7 @@ int lbm_set_step_kernel(lbm_domain* d, int kind, int lz) {
         }
         if (lz > 0) d->tile.push_lz = lz > d->geom.nz ? d->geom.nz : lz;
         d->tile.kind = kind;
+        d->chosen = true;
         drop_graphs(d);
         return fp32 ? ensure_push_maps(d) : ensure_push16_maps(d);
     }
@@ -818,6 +834,7 @@ int lbm_set_step_kernel(lbm_domain* d, int kind, int lz) {
         d->tile.tma_lz = lz <= 0 ? tma_default_lz(d->geom) : (lz > d->geom.nz ? d->geom.nz : lz);
     }
     d->tile.kind = kind;
+    d->chosen = true;
     drop_graphs(d);
     return LBM_OK;
 }
@@ -847,6 +864,7 @@ int lbm_set_push_shape(lbm_domain* d, int shape, int lz) {
     d->tile.push_lz = lz > 0 ? (lz > d->geom.nz ? d->geom.nz : lz)
                              : (fp32 ? push_default_lz(d->geom, shape) : push16_default_lz(d->geom, shape));
     d->tile.kind = LBM_KERNEL_PUSH;
+    d->chosen = true;
     drop_graphs(d);
     return fp32 ? ensure_push_maps(d) : ensure_push16_maps(d);
 }
@@ -890,6 +908,7 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
     const size_t fbytes = (fp32 ? sizeof(float) * 2 : sizeof(uint32_t)) * (size_t)g.plane * Q;
     const size_t rbytes = fp32 ? 0 : sizeof(float2) * (size_t)g.plane;
     const StepTile orig = d->tile;
+    const bool orig_chosen = d->chosen;
     const int cur = d->cur;
     const long long step = d->step;
     const int layout = d->layout;
@@ -961,6 +980,7 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
     };
     auto fail = [&](int code) {
         d->tile = orig;
+        d->chosen = orig_chosen;
         drop_graphs(d);
         if (fsave) restore();
         wait_domain(d);
@@ -983,6 +1003,7 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
     }
     double best = 1e300;
     StepTile best_t = orig;
+    d->chosen = true;  // every candidate is timed as itself
     for (const StepTile& t : cand) {
         d->tile = t;
         drop_graphs(d);

@@ -156,6 +156,11 @@ cudaError_t launch_step2(const float* fin, float* fout, const uint32_t* nbr, con
 cudaError_t launch_step_split(const float* fin, float* fout, float2* rho2, const uint32_t* nbr,
                               const uint32_t* nbr_nw, const uint32_t* adh, const Geom& g, const Phys& p,
                               cudaStream_t s);
+// the same for tau = 1 in both components, on the paired push layout; fin is left
+// with the step's intermediate values (lbm_step_pairs.cu)
+bool pair_step_applicable(const Phys& p);
+cudaError_t launch_step_pairs(float* fin, float* fout, float2* rho2, const uint32_t* nbr, const uint32_t* nbr_nw,
+                              const uint32_t* adh, const Geom& g, const Phys& p, cudaStream_t s);
 // paired push-form step (lbm_step_push.cu): float2 F[19][plane] of the current
 // time level; TMA box loads of whole planes (no periodic x / y, nx even)
 // Inscribed circle of a throat (3 x (cx, cy, cz, r)): the largest clearance
@@ -227,6 +232,7 @@ struct lbm_domain {
     lbmk::Geom geom;
     lbmk::Phys phys;
     lbmk::StepTile tile;
+    bool chosen;        // a step kernel was chosen (lbm_set_tile, _step_kernel, _push_shape, lbm_autotune)
     long long N;
     long long n_fluid;
     float* f[2];       // populations (FP32) or 16-bit deviation pairs (uint32 words)

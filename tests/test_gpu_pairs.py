@@ -1,0 +1,82 @@
+"""The two-launch step at tau = 1 (LBM_KERNEL_SPLIT, and the route of a domain
+without a chosen kernel) against the staged kernel, bit for bit: ragged and odd
+boxes, every periodic axis, boxes one or two cells wide, membrane and reservoirs,
+body force; switching kernels on the way; unequal tau keeps the other two-launch
+kernel.
+"""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+SPHERES = np.array([[9.0, 8.0, 7.0, 5.2], [24.0, 15.0, 19.0, 6.1], [30.5, 3.0, 26.0, 4.0]])
+
+
+@pytest.fixture(scope="module")
+def lbm():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1906_04722_gb300 as m
+    m.load()
+    return m
+
+
+def _domain(lbm, shape, periodic, **par):
+    nz, ny, nx = shape
+    p = lbm.make_params(rho_major=W.RHO_MAJOR, rho_minor=W.RHO_MINOR, periodic=periodic, **par)
+    d = lbm.Domain(p, SPHERES, (nx, ny, nz))
+    d.set_densities(W.droplet_densities(shape, (nx / 2, ny / 2, nz / 2), 0.3 * min(shape) + 1, seed=5))
+    return d
+
+
+def _read(d, steps):
+    d.step(steps)
+    f, st = d.state()
+    return f, st, d.density(), d.measure(allow_nonfinite=True)
+
+
+def _equal(a, b):
+    assert np.array_equal(a[0], b[0]) and a[1] == b[1] and np.array_equal(a[2], b[2])
+    for k in ("n_fluid", "n_w", "n_interface", "n_bulk_w", "n_bulk_nw", "n_in", "n_out", "n_negative"):
+        assert a[3][k] == b[3][k]
+    assert np.allclose(a[3]["mass"], b[3]["mass"], rtol=1e-12, atol=0)
+
+
+@pytest.mark.parametrize("shape,periodic,par", [
+    ((29, 21, 37), (0, 0, 0), {}),
+    ((30, 23, 33), (1, 0, 0), {}),
+    ((31, 20, 34), (0, 1, 1), {"body_force": (1e-5, -2e-5, 3e-5)}),
+    ((16, 17, 18), (1, 1, 1), {"G_ads": (0.0, 0.0)}),
+    ((40, 22, 35), (0, 0, 0), {"reservoirs": True, "membrane_layers": 3}),
+    ((9, 1, 40), (0, 1, 0), {}),
+    ((2, 19, 2), (1, 1, 1), {}),
+])
+def test_equals_the_staged_kernel(lbm, shape, periodic, par):
+    staged = _domain(lbm, shape, periodic, **par)
+    staged.set_step_kernel(lbm.KERNEL_STAGED)
+    want = _read(staged, 70)
+    default = _domain(lbm, shape, periodic, **par)
+    assert default.step_kernel()[0] == lbm.KERNEL_STAGED
+    _equal(_read(default, 70), want)
+    split = _domain(lbm, shape, periodic, **par)
+    split.step(13)
+    split.set_step_kernel(lbm.KERNEL_SPLIT)
+    split.step(30)
+    split.set_step_kernel(lbm.KERNEL_STAGED)
+    split.step(8)
+    split.set_step_kernel(lbm.KERNEL_SPLIT)
+    _equal(_read(split, 19), want)
+
+
+def test_unequal_tau(lbm):
+    a = _domain(lbm, (21, 18, 27), (0, 0, 1), tau=(1.0, 1.2))
+    b = _domain(lbm, (21, 18, 27), (0, 0, 1), tau=(1.0, 1.2))
+    b.set_step_kernel(lbm.KERNEL_STAGED)
+    _equal(_read(a, 20), _read(b, 20))
+    c = _domain(lbm, (21, 18, 27), (0, 0, 1), tau=(1.0, 1.2))
+    c.set_step_kernel(lbm.KERNEL_SPLIT)
+    c.step(20)
+    assert np.allclose(c.density(), a.density(), rtol=1e-5, atol=1e-7)
