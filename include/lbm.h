@@ -617,11 +617,14 @@ int lbm_get_tile(const lbm_domain* d, int* by, int* lz, int* lead);
  *                      density pairs per plane (boxes without periodic x or y
  *                      and with nx % 4 == 0).  Its results equal the staged
  *                      16-bit kernel's bit for bit; the read-outs read
- *                      either layout.
+ *                      either layout.  With tau = 1 in both components and 2^17
+ *                      cells or more the same layout is stepped in two
+ *                      launches, whatever the shape (the same bits).
  * New domains use LBM_KERNEL_STAGED; as long as neither a kernel nor a shape has
- * been chosen, an FP32 domain with tau = 1 in both components steps through the
- * two launches of LBM_KERNEL_SPLIT, with the same bits (lbm_autotune times every kind that applies
- * on the domain).  All give the same results up to rounding (not bit for bit:
+ * been chosen, a domain with tau = 1 in both components steps in two launches
+ * (those of LBM_KERNEL_SPLIT, or their 16-bit counterpart), with the same bits
+ * (lbm_autotune times every kind that applies on the domain, and may leave a 16-bit
+ * domain unchosen).  All give the same results up to rounding (not bit for bit:
  * the TMA kernel folds omega w_k into its equilibrium constants).  LBM_ERR_ARG
  * for an unknown kind, LBM_ERR_STATE when the kernel does not apply to the
  * domain.  lbm_set_tile switches the domain to LBM_KERNEL_STAGED. */

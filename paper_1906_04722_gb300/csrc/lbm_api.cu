@@ -97,18 +97,26 @@ void drop_graphs(lbm_domain* d) {
         }
 }
 
-// Whether steps run as the two launches of lbm_step_pairs.cu: the two-launch kernel
-// at tau = 1, and a domain that nobody has chosen a kernel for -- the results are
-// the staged kernel's bit for bit, and on every box measured it is the faster one
-// (a step of a 32^3 throat 10.4 -> 4.2 us, 48^3 periodic 16.1 -> 7.1 us, the 192^3
-// sample 0.69 -> 0.49 ms).
+// Whether steps run as the two launches of lbm_step_pairs.cu / lbm_step16_pairs.cu
+// (tau = 1 in both components): the two-launch kernel of FP32 domains, a domain that
+// nobody has chosen a kernel for -- the results are the staged kernel's bit for bit,
+// and on every box measured it is the faster one (a step of a 32^3 throat 10.4 -> 4.2
+// us, 48^3 periodic 16.1 -> 7.1 us, the 192^3 sample 0.69 -> 0.49 ms) -- and the push
+// kernel of 16-bit domains from PAIRS16_CELLS cells on (same bits too).
+constexpr long long PAIRS16_CELLS = 1LL << 17;  // 96^3: 75 -> 46 us a step, 192^3: 456 -> 433
 bool steps_in_pairs(const lbm_domain* d) {
-    return d->params.precision == 0 && pair_step_applicable(d->phys) &&
-           (d->tile.kind == LBM_KERNEL_SPLIT || (d->tile.kind == LBM_KERNEL_STAGED && !d->chosen));
+    if (!pair_step_applicable(d->phys)) return false;
+    if (d->tile.kind == LBM_KERNEL_STAGED) return !d->chosen;
+    return d->params.precision == 0 ? d->tile.kind == LBM_KERNEL_SPLIT
+                                    : d->tile.kind == LBM_KERNEL_PUSH && d->N >= PAIRS16_CELLS;
 }
 
 // One step from buffer `cur` to buffer cur ^ 1 on stream s.
 cudaError_t launch_one(lbm_domain* d, int cur, cudaStream_t s) {
+    if (steps_in_pairs(d) && d->params.precision != 0)
+        return launch_step16_pairs(d->params.precision, reinterpret_cast<uint32_t*>(d->f[cur]),
+                                   reinterpret_cast<uint32_t*>(d->f[cur ^ 1]), d->R[cur], d->R[cur ^ 1], d->d_nbr,
+                                   d->d_nbr_nw, d->d_adh, d->geom, d->phys, s);
     if (steps_in_pairs(d))
         return launch_step_pairs(d->f[cur], d->f[cur ^ 1], d->d_rho2, d->d_nbr, d->d_nbr_nw, d->d_adh, d->geom,
                                  d->phys, s);
@@ -914,6 +922,7 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
     const int layout = d->layout;
     // candidates
     std::vector<StepTile> cand;
+    size_t unchosen = SIZE_MAX;  // the candidate that stands for the route of a domain without a chosen kernel
     auto add = [&](int kind, int by, int lz, int lead) {
         StepTile t = orig;
         t.kind = kind;
@@ -948,6 +957,15 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
                 t.push_order = 0;
                 cand.push_back(t);
             }
+    if (!fp32 && pair_step_applicable(d->phys)) {  // reachable in no other way on a small 16-bit box
+        unchosen = cand.size();
+        StepTile t = default_tile(g);
+        t.push_shape = orig.push_shape;
+        t.push_lz = orig.push_lz;
+        t.push_pf = orig.push_pf;
+        t.push_order = orig.push_order;
+        cand.push_back(t);
+    }
     if (fp32 && d->tma_ok)
         for (int lz : {8, 12, 16, 24, 32, 48}) add(LBM_KERNEL_TMA, orig.by, lz, orig.lead);
     if (fp32) add(LBM_KERNEL_SPLIT, orig.by, orig.lz, orig.lead);
@@ -1003,9 +1021,10 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
     }
     double best = 1e300;
     StepTile best_t = orig;
-    d->chosen = true;  // every candidate is timed as itself
+    bool best_chosen = true;
     for (const StepTile& t : cand) {
         d->tile = t;
+        d->chosen = (size_t)(&t - cand.data()) != unchosen;  // timed as itself
         drop_graphs(d);
         if ((rc = restore())) return fail(rc);
         if ((rc = run_steps(d, 1))) return fail(rc);  // untimed: kernel set-up, ghost stores
@@ -1019,9 +1038,11 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
         if (per < best) {
             best = per;
             best_t = t;
+            best_chosen = d->chosen;
         }
     }
     d->tile = best_t;
+    d->chosen = best_chosen;
     drop_graphs(d);
     if ((rc = restore())) return fail(rc);
     rc = wait_domain(d);

@@ -161,6 +161,10 @@ cudaError_t launch_step_split(const float* fin, float* fout, float2* rho2, const
 bool pair_step_applicable(const Phys& p);
 cudaError_t launch_step_pairs(float* fin, float* fout, float2* rho2, const uint32_t* nbr, const uint32_t* nbr_nw,
                               const uint32_t* adh, const Geom& g, const Phys& p, cudaStream_t s);
+// the same for 16-bit storage, on its push layout (lbm_step16_pairs.cu)
+cudaError_t launch_step16_pairs(int precision, uint32_t* win, uint32_t* wout, const float2* Rin, float2* Rout,
+                                const uint32_t* nbr, const uint32_t* nbr_nw, const uint32_t* adh, const Geom& g,
+                                const Phys& p, cudaStream_t s);
 // paired push-form step (lbm_step_push.cu): float2 F[19][plane] of the current
 // time level; TMA box loads of whole planes (no periodic x / y, nx even)
 // Inscribed circle of a throat (3 x (cx, cy, cz, r)): the largest clearance

@@ -80,3 +80,38 @@ def test_unequal_tau(lbm):
     c.set_step_kernel(lbm.KERNEL_SPLIT)
     c.step(20)
     assert np.allclose(c.density(), a.density(), rtol=1e-5, atol=1e-7)
+
+
+@pytest.mark.parametrize("precision", [1, 2])
+@pytest.mark.parametrize("shape,periodic,par", [
+    ((29, 21, 37), (0, 0, 0), {}),
+    ((31, 20, 34), (1, 1, 1), {"body_force": (1e-5, -2e-5, 3e-5)}),
+    ((40, 22, 35), (0, 0, 0), {"reservoirs": True, "membrane_layers": 3}),
+    ((2, 19, 2), (1, 1, 1), {}),
+    ((52, 51, 52), (0, 0, 1), {}),
+    ((101, 102, 104), (0, 0, 0), {"reservoirs": True, "membrane_layers": 2}),
+])
+def test_16_bit(lbm, precision, shape, periodic, par):
+    """Untuned, and (from 2^17 cells on) as the push kernel; the last box is one
+    of 2^20 cells and more, whose second launch reads the densities twice."""
+    staged = _domain(lbm, shape, periodic, precision=precision, **par)
+    staged.set_step_kernel(lbm.KERNEL_STAGED)
+    default = _domain(lbm, shape, periodic, precision=precision, **par)
+    push = _domain(lbm, shape, periodic, precision=precision, **par)
+    for d in (staged, default):
+        d.step(31)
+    if shape[2] % 4 == 0 and not periodic[0]:
+        push.step(9)
+        push.set_step_kernel(lbm.KERNEL_PUSH)
+        push.step(11)
+        push.set_step_kernel(lbm.KERNEL_STAGED)
+        push.step(5)
+        push.set_push_shape(0, 8)
+        push.step(6)
+    else:
+        push.step(31)
+    for d in (default, push):
+        assert np.array_equal(d.density(), staged.density())
+        a, b = d.measure(allow_nonfinite=True), staged.measure(allow_nonfinite=True)
+        assert a["n_w"] == b["n_w"] and a["n_interface"] == b["n_interface"]
+        assert d.density_at(1, 5, 1) == staged.density_at(1, 5, 1)
