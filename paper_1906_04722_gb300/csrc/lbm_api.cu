@@ -111,12 +111,23 @@ bool steps_in_pairs(const lbm_domain* d) {
                                     : d->tile.kind == LBM_KERNEL_PUSH && d->N >= PAIRS16_CELLS;
 }
 
-// One step from buffer `cur` to buffer cur ^ 1 on stream s.
+// Whether such a domain's steps run on moments (lbm_step_moments.cu), in place in one
+// population buffer.
+#ifndef MOMENT_CELLS
+#define MOMENT_CELLS 0
+#endif
+bool steps_on_moments(const lbm_domain* d) {
+    return d->params.precision == 0 && steps_in_pairs(d) && d->N >= MOMENT_CELLS;
+}
+
+// One step from buffer `cur` to buffer cur ^ 1 (on moments: in place) on stream s.
 cudaError_t launch_one(lbm_domain* d, int cur, cudaStream_t s) {
     if (steps_in_pairs(d) && d->params.precision != 0)
         return launch_step16_pairs(d->params.precision, reinterpret_cast<uint32_t*>(d->f[cur]),
                                    reinterpret_cast<uint32_t*>(d->f[cur ^ 1]), d->R[cur], d->R[cur ^ 1], d->d_nbr,
                                    d->d_nbr_nw, d->d_adh, d->geom, d->phys, s);
+    if (steps_on_moments(d))
+        return launch_step_moments(d->f[cur], d->d_nbr, d->d_nbr_nw, d->d_adh, d->geom, d->phys, s);
     if (steps_in_pairs(d))
         return launch_step_pairs(d->f[cur], d->f[cur ^ 1], d->d_rho2, d->d_nbr, d->d_nbr_nw, d->d_adh, d->geom,
                                  d->phys, s);
@@ -158,10 +169,26 @@ cudaError_t prepare_one(lbm_domain* d) {
 // pull words, each at its reader), every other kernel in the pull layout.
 int wanted_layout(const lbm_domain* d) { return d->tile.kind == LBM_KERNEL_PUSH || steps_in_pairs(d) ? 1 : 0; }
 
+// Clears the buffer that is not current.  In the pull layout the slots of grain cells
+// hold 0 (a checkpoint shows them) and the step kernels never write them: what
+// another layout left there goes before the buffer is stepped into.
+int clear_other(lbm_domain* d) {
+    const size_t bytes = (d->params.precision == 0 ? sizeof(float) * 2 : sizeof(uint32_t)) * (size_t)d->geom.plane * Q;
+    LBM_CUDA(cudaMemsetAsync(d->f[d->cur ^ 1], 0, bytes, d->stream));
+    return LBM_OK;
+}
+
 // Converts the state into the given layout (into the other buffer, which then
 // becomes the current one).  The step counter is unchanged.
 int set_layout(lbm_domain* d, int layout) {
     if (d->layout == layout) return LBM_OK;
+    if (d->layout == 2) {
+        LBM_CUDA(launch_moments_to_pull(d->f[d->cur], d->f[d->cur ^ 1], d->d_nbr, d->geom, d->stream));
+        d->cur ^= 1;
+        d->layout = 0;
+        d->ghosts_ok = false;
+        if (layout == 0) return clear_other(d);
+    }
     if (d->params.precision != 0) {
         const uint32_t* in = reinterpret_cast<const uint32_t*>(d->f[d->cur]);
         uint32_t* out = reinterpret_cast<uint32_t*>(d->f[d->cur ^ 1]);
@@ -181,18 +208,21 @@ int set_layout(lbm_domain* d, int layout) {
     d->cur ^= 1;
     d->layout = layout;
     d->ghosts_ok = false;
-    return LBM_OK;
+    return layout == 0 ? clear_other(d) : LBM_OK;
 }
 
 // The current FP32 state in the pull layout, for the read-out kernels: f[cur]
-// itself, or (paired push layout) its conversion into the other buffer, which
+// itself, or (another layout) its conversion into the other buffer, which
 // the next step overwrites anyway.
 int pull_view(lbm_domain* d, const float** out) {
     if (d->layout == 0) {
         *out = d->f[d->cur];
         return LBM_OK;
     }
-    LBM_CUDA(launch_push_to_pull(d->f[d->cur], d->f[d->cur ^ 1], d->d_nbr, d->d_nbr_nw, d->geom, d->stream));
+    if (d->layout == 2)
+        LBM_CUDA(launch_moments_to_pull(d->f[d->cur], d->f[d->cur ^ 1], d->d_nbr, d->geom, d->stream));
+    else
+        LBM_CUDA(launch_push_to_pull(d->f[d->cur], d->f[d->cur ^ 1], d->d_nbr, d->d_nbr_nw, d->geom, d->stream));
     *out = d->f[d->cur ^ 1];
     return LBM_OK;
 }
@@ -238,7 +268,7 @@ int capture_graph(lbm_domain* d, int parity) {
     cudaError_t err = cudaSuccess;
     for (int i = 0; i < GRAPH_STEPS && err == cudaSuccess; ++i) {
         err = launch_one(d, cur, d->capture_stream);
-        cur ^= 1;
+        if (!steps_on_moments(d)) cur ^= 1;
     }
     cudaGraph_t graph = nullptr;
     cudaError_t end = cudaStreamEndCapture(d->capture_stream, &graph);
@@ -261,7 +291,17 @@ int capture_graph(lbm_domain* d, int parity) {
 // n steps: whole chunks replay a captured graph, the remainder is launched one by one.
 int run_steps(lbm_domain* d, int n) {
     if (n <= 0) return LBM_OK;
-    if (int rc = set_layout(d, wanted_layout(d))) return rc;
+    const bool moments = steps_on_moments(d);
+    if (!moments || d->layout != 2)
+        if (int rc = set_layout(d, wanted_layout(d))) return rc;
+    if (moments && d->layout != 2) {  // any state: one step from the populations builds the moments
+        LBM_CUDA(launch_first_moments(d->f[d->cur], d->d_rho2, d->f[d->cur ^ 1], d->d_nbr, d->d_adh, d->geom, d->phys,
+                                      d->stream));
+        d->cur ^= 1;
+        d->layout = 2;
+        ++d->step;
+        --n;
+    }
     if (d->tile.kind == LBM_KERNEL_PUSH) {
         if (int rc = d->params.precision == 0 ? ensure_push_maps(d) : ensure_push16_maps(d)) return rc;
         d->tma_pending = true;  // the push kernels report a wait that ran out through d_err
@@ -285,7 +325,7 @@ int run_steps(lbm_domain* d, int n) {
     for (int i = 0; i < n; ++i) {
         LBM_CUDA(prepare_one(d));
         LBM_CUDA(launch_one(d, d->cur, d->stream));
-        d->cur ^= 1;
+        if (!moments) d->cur ^= 1;
         ++d->step;
     }
     return LBM_OK;
@@ -386,10 +426,13 @@ int init_from_densities(lbm_domain* d) {
         LBM_CUDA(cudaMemsetAsync(d->f[0], 0, sizeof(uint32_t) * (size_t)d->geom.plane * Q, d->stream));
         LBM_CUDA(launch_init16(d->d_rho, d->R[0], d->geom, d->stream));
     }
+    const bool dirty = d->layout != 0;
     d->cur = 0;
     d->step = 0;
     d->ghosts_ok = false;
     d->layout = 0;
+    if (dirty)
+        if (int rc = clear_other(d)) return rc;
     return wait_domain(d);
 }
 
@@ -408,7 +451,10 @@ int upload_densities(lbm_domain* d, const double* rho) {
 // Queue the measurement of the current state, its sums going to h_result; after a
 // wait, read_measurement gives the observables.
 int queue_measure(lbm_domain* d) {
-    if (d->params.precision == 0 && d->layout == 1) {
+    if (d->layout == 2) {
+        LBM_CUDA(launch_measure_moments(d->f[d->cur], d->d_rho2, d->d_nbr, d->d_nbr_nw, d->geom, d->params.G,
+                                        d->d_partials, d->meas_blocks, d->d_result, d->stream));
+    } else if (d->params.precision == 0 && d->layout == 1) {
         LBM_CUDA(launch_measure_push(d->f[d->cur], d->d_nbr, d->geom, d->params.G, d->d_partials, d->meas_blocks,
                                      d->d_result, d->stream));
     } else if (d->params.precision == 0) {
@@ -461,7 +507,9 @@ int queue_probe(lbm_domain* d, int x, int y, int z) {
         set_error("probe cell outside the box");
         return LBM_ERR_ARG;
     }
-    if (d->params.precision == 0 && d->layout == 1) {
+    if (d->layout == 2) {
+        LBM_CUDA(launch_probe_moments(d->f[d->cur], d->d_nbr, d->d_nbr_nw, d->geom, x, y, z, d->d_probe, d->stream));
+    } else if (d->params.precision == 0 && d->layout == 1) {
         LBM_CUDA(launch_probe_push(d->f[d->cur], d->d_nbr, d->geom, x, y, z, d->d_probe, d->stream));
     } else if (d->params.precision == 0) {
         LBM_CUDA(launch_probe(d->f[d->cur], d->d_nbr, d->d_nbr_nw, d->geom, x, y, z, d->d_probe, d->stream));
@@ -724,7 +772,10 @@ int lbm_measure(lbm_domain* d, lbm_measurement* out) {
 int lbm_get_density(lbm_domain* d, double* rho_out) {
     if (!d || !rho_out) { set_error("domain or rho_out is NULL"); return LBM_ERR_ARG; }
     try {
-        if (d->params.precision == 0 && d->layout == 1) {
+        if (d->layout == 2) {
+            LBM_CUDA(launch_density_moments(d->f[d->cur], d->d_rho2, d->d_rho, d->d_nbr, d->d_nbr_nw, d->geom,
+                                            d->stream));
+        } else if (d->params.precision == 0 && d->layout == 1) {
             LBM_CUDA(launch_density_push(d->f[d->cur], d->d_nbr, d->geom, d->d_rho, d->stream));
         } else if (d->params.precision == 0) {
             LBM_CUDA(launch_density(d->f[d->cur], d->d_rho, d->d_nbr, d->d_nbr_nw, d->geom, d->stream));
@@ -784,9 +835,12 @@ int lbm_set_state(lbm_domain* d, const float* f_in, long long step) {
     for (int p = 0; p < 2 * Q; ++p)
         LBM_CUDA(cudaMemcpyAsync(d->f[d->cur] + (size_t)p * d->geom.plane, f_in + (size_t)p * N, sizeof(float) * N,
                                  cudaMemcpyHostToDevice, d->stream));
+    const bool dirty = d->layout != 0;
     d->step = step;
     d->ghosts_ok = false;
     d->layout = 0;
+    if (dirty)
+        if (int rc = clear_other(d)) return rc;
     return wait_domain(d);
 }
 
@@ -1045,6 +1099,8 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
     d->chosen = best_chosen;
     drop_graphs(d);
     if ((rc = restore())) return fail(rc);
+    if (d->layout == 0)
+        if ((rc = clear_other(d))) return fail(rc);
     rc = wait_domain(d);
     cleanup();
     if (rc) return rc;

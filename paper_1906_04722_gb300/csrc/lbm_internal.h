@@ -161,6 +161,24 @@ cudaError_t launch_step_split(const float* fin, float* fout, float2* rho2, const
 bool pair_step_applicable(const Phys& p);
 cudaError_t launch_step_pairs(float* fin, float* fout, float2* rho2, const uint32_t* nbr, const uint32_t* nbr_nw,
                               const uint32_t* adh, const Geom& g, const Phys& p, cudaStream_t s);
+// its first launch alone
+cudaError_t launch_pair_moments(float* F, float2* rho2, const uint32_t* nbr, const Geom& g, cudaStream_t s);
+// tau = 1 in both components on moments, in place in one population buffer
+// (lbm_step_moments.cu); the first step starts from the paired push layout F (left
+// with intermediate values) and builds the moments in `buffer`
+cudaError_t launch_step_moments(float* buffer, const uint32_t* nbr, const uint32_t* nbr_nw, const uint32_t* adh,
+                                const Geom& g, const Phys& p, cudaStream_t s);
+cudaError_t launch_first_moments(float* F, float2* rho2, float* buffer, const uint32_t* nbr, const uint32_t* adh,
+                                 const Geom& g, const Phys& p, cudaStream_t s);
+cudaError_t launch_moments_to_pull(float* buffer, float* fout, const uint32_t* nbr, const Geom& g, cudaStream_t s);
+// read-outs of a state on moments (rho2: scratch of one pair per cell)
+cudaError_t launch_density_moments(float* buffer, float2* rho2, float* rho, const uint32_t* nbr, const uint32_t* nbr_nw,
+                                   const Geom& g, cudaStream_t s);
+cudaError_t launch_measure_moments(float* buffer, float2* rho2, const uint32_t* nbr, const uint32_t* nbr_nw,
+                                   const Geom& g, double G, double* partials, int nblocks, double* result,
+                                   cudaStream_t s);
+cudaError_t launch_probe_moments(float* buffer, const uint32_t* nbr, const uint32_t* nbr_nw, const Geom& g, int x,
+                                 int y, int z, float* out, cudaStream_t s);
 // the same for 16-bit storage, on its push layout (lbm_step16_pairs.cu)
 cudaError_t launch_step16_pairs(int precision, uint32_t* win, uint32_t* wout, const float2* Rin, float2* Rout,
                                 const uint32_t* nbr, const uint32_t* nbr_nw, const uint32_t* adh, const Geom& g,
@@ -268,7 +286,7 @@ struct lbm_domain {
     int* h_err;         // pinned copy of d_err, read after a wait
     bool tma_pending;   // a TMA step ran since d_err was last read
     float2* d_rho2;     // FP32 domains: (rho_w, rho_nw) per cell for the two-launch step
-    int layout;         // FP32 state in f[cur]: 0 = pull layout, 1 = paired push layout
+    int layout;         // state in f[cur]: 0 = pull layout, 1 = push layout (FP32: paired), 2 = moments (FP32, tau = 1)
     CUtensorMap push_maps[2];  // tensor maps of f[0], f[1] for the push kernel's shape
     CUtensorMap push16_w[2];   // 16-bit storage: tensor maps of the words of f[0], f[1]
     CUtensorMap push16_r[2];   // and of the density pairs R[0], R[1]

@@ -110,12 +110,18 @@ __global__ void __launch_bounds__(PAIR_THREADS, 8)
 
 bool pair_step_applicable(const Phys& p) { return p.tau[0] == 1.0f && p.tau[1] == 1.0f; }
 
+cudaError_t launch_pair_moments(float* F, float2* rho2, const uint32_t* nbr, const Geom& g, cudaStream_t s) {
+    const int N = g.nxy * g.nz;
+    pair_moment_kernel<<<(unsigned)((N + PAIR_THREADS - 1) / PAIR_THREADS), PAIR_THREADS, 0, s>>>(
+        reinterpret_cast<float2*>(F), rho2, nbr, g, N);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_step_pairs(float* fin, float* fout, float2* rho2, const uint32_t* nbr, const uint32_t* nbr_nw,
                               const uint32_t* adh, const Geom& g, const Phys& p, cudaStream_t s) {
     const int N = g.nxy * g.nz;
     const unsigned blocks = (unsigned)((N + PAIR_THREADS - 1) / PAIR_THREADS);
-    pair_moment_kernel<<<blocks, PAIR_THREADS, 0, s>>>(reinterpret_cast<float2*>(fin), rho2, nbr, g, N);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_pair_moments(fin, rho2, nbr, g, s);
     if (e != cudaSuccess) return e;
     pair_push_kernel<<<blocks, PAIR_THREADS, 0, s>>>(reinterpret_cast<const float2*>(fin),
                                                     reinterpret_cast<float2*>(fout), rho2, nbr, nbr_nw, adh, g, p, N);
