@@ -589,8 +589,10 @@ int lbm_get_tile(const lbm_domain* d, int* by, int* lz, int* lead);
  *                      densities from it (any box; FP32 only; lz ignored); with
  *                      tau = 1 in both components on the paired push layout
  *                      below, the second launch working from densities and
- *                      velocities alone (the staged kernel's results bit for
- *                      bit);
+ *                      velocities alone, and on large boxes with the state kept
+ *                      as each cell's densities, equilibrium velocities and rest
+ *                      populations, from which its neighbours' populations are
+ *                      formed (the staged kernel's results bit for bit);
  *   LBM_KERNEL_STAGED2 the staged kernel with two threads per cell, one per
  *                      fluid component (any box; FP32 only; by 6 or 8, lead 2,
  *                      lz planes per z segment, lz <= 0: keep the current).

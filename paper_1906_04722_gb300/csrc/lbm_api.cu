@@ -9,6 +9,7 @@
 #include <thread>
 #include <vector>
 
+#include "lbm_host.h"
 #include "lbm_internal.h"
 
 namespace lbmk {
@@ -101,8 +102,8 @@ void drop_graphs(lbm_domain* d) {
 // (tau = 1 in both components): the two-launch kernel of FP32 domains, a domain that
 // nobody has chosen a kernel for -- the results are the staged kernel's bit for bit,
 // and on every box measured it is the faster one (a step of a 32^3 throat 10.4 -> 4.2
-// us, 48^3 periodic 16.1 -> 7.1 us, the 192^3 sample 0.69 -> 0.49 ms) -- and the push
-// kernel of 16-bit domains from PAIRS16_CELLS cells on (same bits too).
+// us, 48^3 periodic 16.1 -> 7.1 us, the 192^3 sample 0.69 -> 0.32 ms on moments) -- and
+// the push kernel of 16-bit domains from PAIRS16_CELLS cells on (same bits too).
 constexpr long long PAIRS16_CELLS = 1LL << 17;  // 96^3: 75 -> 46 us a step, 192^3: 456 -> 433
 bool steps_in_pairs(const lbm_domain* d) {
     if (!pair_step_applicable(d->phys)) return false;
@@ -112,10 +113,11 @@ bool steps_in_pairs(const lbm_domain* d) {
 }
 
 // Whether such a domain's steps run on moments (lbm_step_moments.cu), in place in one
-// population buffer.
-#ifndef MOMENT_CELLS
-#define MOMENT_CELLS 0
-#endif
+// population buffer: from the size on where the two population buffers (304 bytes a
+// cell) have outgrown the 129 MB L2 by a half.  On moments against on pairs: 80^3
+// 29.7 against 21.3 us a step, 96^3 40 against 56, 112 x 97 x 120 70 against 89, 192^3
+// 319 against 492.
+constexpr long long MOMENT_CELLS = 5LL << 17;
 bool steps_on_moments(const lbm_domain* d) {
     return d->params.precision == 0 && steps_in_pairs(d) && d->N >= MOMENT_CELLS;
 }
@@ -785,6 +787,7 @@ int lbm_get_density(lbm_domain* d, double* rho_out) {
                                       d->R[d->cur], d->d_nbr, d->d_nbr_nw, d->geom, d->layout == 1, d->d_rho,
                                       d->stream));
         }
+        touch_pages(rho_out, sizeof(double) * 2 * (size_t)d->N);
         for (long long i = 0; i < 2 * d->N; i += CONVERT_PIECE) {
             const long long n = std::min(CONVERT_PIECE, 2 * d->N - i);
             to_double_kernel<<<1216, 256, 0, d->stream>>>(d->d_rho + i, d->d_convert, n);
@@ -819,6 +822,7 @@ int lbm_get_state(lbm_domain* d, float* f_out, long long* step_out) {
     const long long N = d->N;
     const float* fp = nullptr;
     if (int rc = pull_view(d, &fp)) return rc;
+    touch_pages(f_out, sizeof(float) * 2 * Q * (size_t)N);
     for (int p = 0; p < 2 * Q; ++p)
         LBM_CUDA(cudaMemcpyAsync(f_out + (size_t)p * N, fp + (size_t)p * d->geom.plane, sizeof(float) * N,
                                  cudaMemcpyDeviceToHost, d->stream));

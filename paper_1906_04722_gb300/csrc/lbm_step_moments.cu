@@ -7,38 +7,41 @@
 // computed from its neighbours' moments, with the very operations that would have
 // stored them (pair_equilibrium's, one direction at a time), and agree bit for bit.
 //
-//   moment_gather_kernel   reads the neighbours' moments (rs, u, base, rest), forms
+//   moment_gather_kernel   reads the neighbours' moments (rs, base, u, rest), forms
 //                          the 19 incoming pairs, and stores the cell's densities
 //                          and common velocity (20 bytes);
 //   moment_collide_kernel  reads those and the neighbours' densities and stores the
 //                          cell's new moments (48 bytes).
 //
 // Each launch reads what the other wrote, so one copy of the state is enough; it
-// lies in one population buffer.  DRAM moves about 140 bytes a cell and step, where
-// a step on populations moves 304 plus what its tiles re-read; the price is
-// arithmetic (each direction's equilibrium is formed by its reader, without the
-// sharing between opposite directions) and loads, which L1 and L2 serve: a CTA is a
-// 32 x 2 x 2 brick.
+// lies in one population buffer.  DRAM moves about 0.9 GB a step of the 192^3 sample,
+// where the tuned push kernel moves 2.1; the price is arithmetic (each direction's
+// equilibrium is formed by its reader, without the sharing between opposite
+// directions) and loads, which L1 and L2 serve.  Bound by the latency of those
+// loads: a CTA is a 32 x 4 x 2 brick, six to an SM (40 registers a thread), and a
+// cell's densities and u^2 term come in one 16-byte load.  192^3: 319 us a step (420
+// push kernel, 492 on pairs); bricks of 32 x 2 x 2 at eight an SM (64 registers) 370,
+// 32 x 4 x 1 at twelve 321, 32 x 8 x 2 at two 389.
 #include "lbm_collide_pair.cuh"
 
 namespace lbmk {
 
 namespace {
 
-constexpr int MX = 32, MY = 2, MZ = 2, MT = MX * MY * MZ;
+constexpr int MX = 32, MY = 4, MZ = 2, MT = MX * MY * MZ;
 
 // Arrays of the state in a population buffer, `plane` pairs apart.
 struct Moments {
-    float2 *rs, *u[3], *base, *rest;  // equilibrium density and velocity, rs (1 - 1.5 u^2), rest pair
-    float2 *rho, *upxy;               // densities of the cells and their common velocity
+    float4* rb;          // equilibrium densities rs and rs (1 - 1.5 u^2), the components side by side
+    float2 *u[3], *rest;  // equilibrium velocity, rest pair
+    float2 *rho, *upxy;   // densities of the cells and their common velocity
     float* upz;
 };
 __host__ __device__ __forceinline__ Moments moments_in(float* buffer, int plane) {
     float2* b = reinterpret_cast<float2*>(buffer);
     Moments m;
-    m.rs = b;
-    for (int d = 0; d < 3; ++d) m.u[d] = b + (size_t)(1 + d) * plane;
-    m.base = b + (size_t)4 * plane;
+    m.rb = reinterpret_cast<float4*>(buffer);
+    for (int d = 0; d < 3; ++d) m.u[d] = b + (size_t)(2 + d) * plane;
     m.rest = b + (size_t)5 * plane;
     m.rho = b + (size_t)6 * plane;
     m.upxy = b + (size_t)7 * plane;
@@ -69,7 +72,8 @@ struct Cell {
 // What cell s sends in direction k (reversed: in direction opposite to k).
 __device__ __forceinline__ float2 sent(const Moments& m, int s, int k, bool reversed) {
     const int o = k & 1 ? k : k - 1;  // the odd direction of the pair
-    const float2 r = __ldg(m.rs + s), base = __ldg(m.base + s);
+    const float4 rb = __ldg(m.rb + s);
+    const float2 r = make_float2(rb.x, rb.y), base = make_float2(rb.z, rb.w);
     const float2 ux = EX(o) ? __ldg(m.u[0] + s) : make_float2(0.f, 0.f);
     const float2 uy = EY(o) ? __ldg(m.u[1] + s) : make_float2(0.f, 0.f);
     const float2 uz = EZ(o) ? __ldg(m.u[2] + s) : make_float2(0.f, 0.f);
@@ -106,7 +110,7 @@ __device__ __forceinline__ bool my_cell(const Geom& g, int& x, int& y, int& z) {
     return x < g.nx && y < g.ny && z < g.nz;
 }
 
-__global__ void __launch_bounds__(MT, 8)
+__global__ void __launch_bounds__(MT, 6)
     moment_gather_kernel(float* buffer, const uint32_t* __restrict__ nbr, const uint32_t* __restrict__ nbr_nw, Geom g) {
     int x, y, z;
     if (!my_cell(g, x, y, z)) return;
@@ -134,7 +138,7 @@ __global__ void __launch_bounds__(MT, 8)
 // FIRST: the densities and common velocity come from a step that started on
 // populations (pair_moment_kernel: rho2, and two of the cell's slots in F).
 template <bool FIRST>
-__global__ void __launch_bounds__(MT, 8)
+__global__ void __launch_bounds__(MT, 6)
     moment_collide_kernel(float* buffer, const float2* __restrict__ F, const float2* __restrict__ rho2,
                           const uint32_t* __restrict__ nbr, const uint32_t* __restrict__ adh, Geom g, Phys P) {
     int x, y, z;
@@ -168,10 +172,10 @@ __global__ void __launch_bounds__(MT, 8)
     if (!open_end) rest = sum;
     // pair_equilibrium's own u^2 and base
     const float2 uu = pfma(u[2], u[2], pfma(u[0], u[0], pmul(u[1], u[1])));
-    m.rs[at.c] = r;
+    const float2 base = pmul(r, pfma(pair2(-1.5f), uu, pair2(1.f)));
+    m.rb[at.c] = make_float4(r.x, r.y, base.x, base.y);
 #pragma unroll
     for (int d = 0; d < 3; ++d) m.u[d][at.c] = u[d];
-    m.base[at.c] = pmul(r, pfma(pair2(-1.5f), uu, pair2(1.f)));
     m.rest[at.c] = rest;
 }
 
@@ -237,7 +241,7 @@ __global__ void __launch_bounds__(MT)
     const Moments m = moments_in(buffer, g.plane);
     const bool fluid = cls != CLS_SOLID, has_nw = fluid && cls != CLS_MEMBRANE;
     const float2 zero = make_float2(0.f, 0.f);
-    const float2 r = fluid ? m.rs[c] : zero, rest = fluid ? m.rest[c] : zero;
+    const float2 r = fluid ? make_float2(m.rb[c].x, m.rb[c].y) : zero, rest = fluid ? m.rest[c] : zero;
     const float2 u[3] = {fluid ? m.u[0][c] : zero, fluid ? m.u[1][c] : zero, fluid ? m.u[2][c] : zero};
     auto put = [&](int k, float2 v) {
         fout[(size_t)k * g.plane + c] = fluid ? v.x : 0.f;

@@ -13,7 +13,7 @@
 // 1.16 GB are whole rows with their grain) and the second, which waits on its
 // scattered 8-byte stores (47 M partial sectors for 25 M), takes 0.30 ms at 3.8
 // TB/s: 0.49 ms a step against 0.42 of the tuned push kernel and 0.69 of the staged
-// one.  Any box and any periodic axes; results equal the staged kernel's bit for bit.
+// one; boxes of that size step on moments (lbm_step_moments.cu).  Any box and any periodic axes; results equal the staged kernel's bit for bit.
 #include "lbm_collide_pair.cuh"
 
 namespace lbmk {
