@@ -983,8 +983,6 @@ int lbm_surrogate_predict(lbm_surrogate* s, const float* X, int n, float* mean, 
     cudaError_t e;
     if ((e = cudaMalloc(&dMean, sizeof(float) * (size_t)chunk * nout)) != cudaSuccess) { cleanup(); return sur_fail(e, "cudaMalloc"); }
     if ((e = cudaMalloc(&dSpread, sizeof(float) * (size_t)chunk * nout)) != cudaSuccess) { cleanup(); return sur_fail(e, "cudaMalloc"); }
-    touch_pages(mean, sizeof(float) * (size_t)n * nout);
-    touch_pages(spread, sizeof(float) * (size_t)n * nout);
     for (int r0 = 0; r0 < n; r0 += chunk) {
         const int rows = std::min(chunk, n - r0);
         if ((e = cudaMemcpyAsync(act(s, 0, 0), X + (size_t)r0 * nin, sizeof(float) * rows * nin, cudaMemcpyHostToDevice,
