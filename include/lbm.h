@@ -127,7 +127,8 @@ int lbm_set_pressure_bc(lbm_domain* d, double rho_in_nw, double rho_out_w);
 /* lbm_step -- queue n_steps fused time steps on the domain's stream
  * (asynchronous; n_steps >= 0).  Whole chunks of 64 steps replay a CUDA graph
  * captured on first use (one per starting buffer, recaptured after
- * lbm_set_tile); the remainder is launched step by step.  Results are the same
+ * lbm_set_tile), chunks of 8 another one once the domain has been stepped in short
+ * runs a few times; the remainder is launched step by step.  Results are the same
  * either way, bit for bit. */
 int lbm_step(lbm_domain* d, int n_steps);
 

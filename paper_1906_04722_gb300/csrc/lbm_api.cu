@@ -1,6 +1,7 @@
 // lbm_api.cu -- the extern "C" entry points declared in include/lbm.h.
 #include <algorithm>
 #include <chrono>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -91,11 +92,13 @@ int set_bc(lbm_domain* d, double rho_in_nw, double rho_out_w) {
 }
 
 void drop_graphs(lbm_domain* d) {
-    for (int i = 0; i < 2; ++i)
-        if (d->graph[i]) {
-            cudaGraphExecDestroy(d->graph[i]);
-            d->graph[i] = nullptr;
-        }
+    for (auto& of_parity : d->graph)
+        for (cudaGraphExec_t& g : of_parity)
+            if (g) {
+                cudaGraphExecDestroy(g);
+                g = nullptr;
+            }
+    d->short_runs = std::min(d->short_runs, 0);  // counted anew; below 0: lbm_autotune is timing
 }
 
 // Whether steps run as the two launches of lbm_step_pairs.cu / lbm_step16_pairs.cu
@@ -260,15 +263,15 @@ int ensure_push_maps(lbm_domain* d) {
     return LBM_OK;
 }
 
-// Capture GRAPH_STEPS step launches that start from buffer `parity` on the
+// Capture GRAPH_STEPS[size] step launches that start from buffer `parity` on the
 // domain's private capture stream; the graph is launched on the domain's stream.
-int capture_graph(lbm_domain* d, int parity) {
+int capture_graph(lbm_domain* d, int parity, int size) {
     LBM_CUDA(prepare_one(d));
     if (!d->capture_stream) LBM_CUDA(cudaStreamCreateWithFlags(&d->capture_stream, cudaStreamNonBlocking));
     LBM_CUDA(cudaStreamBeginCapture(d->capture_stream, cudaStreamCaptureModeThreadLocal));
     int cur = parity;
     cudaError_t err = cudaSuccess;
-    for (int i = 0; i < GRAPH_STEPS && err == cudaSuccess; ++i) {
+    for (int i = 0; i < GRAPH_STEPS[size] && err == cudaSuccess; ++i) {
         err = launch_one(d, cur, d->capture_stream);
         if (!steps_on_moments(d)) cur ^= 1;
     }
@@ -280,17 +283,24 @@ int capture_graph(lbm_domain* d, int parity) {
                   cudaGetErrorString(err != cudaSuccess ? err : end));
         return LBM_ERR_CUDA;
     }
-    cudaError_t inst = cudaGraphInstantiate(&d->graph[parity], graph, 0);
+    cudaError_t inst = cudaGraphInstantiate(&d->graph[parity][size], graph, 0);
     cudaGraphDestroy(graph);
     if (inst != cudaSuccess) {
-        d->graph[parity] = nullptr;
+        d->graph[parity][size] = nullptr;
         set_error(std::string("cudaGraphInstantiate: ") + cudaGetErrorString(inst));
         return LBM_ERR_CUDA;
     }
     return LBM_OK;
 }
 
-// n steps: whole chunks replay a captured graph, the remainder is launched one by one.
+bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+    cudaGetLastError();  // the legacy stream while another stream captures
+    return true;
+}
+
+// n steps: whole chunks replay captured graphs, the remainder is launched one by one.
 int run_steps(lbm_domain* d, int n) {
     if (n <= 0) return LBM_OK;
     const bool moments = steps_on_moments(d);
@@ -315,14 +325,20 @@ int run_steps(lbm_domain* d, int n) {
     }
     if (!tma) d->ghosts_ok = false;
     if (tma) d->tma_pending = true;
-    while (n >= GRAPH_STEPS) {
-        if (!d->graph[d->cur]) {
-            int rc = capture_graph(d, d->cur);
-            if (rc) return rc;
+    // Chunks of 64 steps replay a graph, and so do chunks of 8 once a domain has been
+    // stepped in short runs a few times (a capture costs about what it saves in two
+    // or three such runs); not while a caller captures the domain's stream.  A 32^3
+    // throat's ladder of 20 x 25 two-launch steps is bound by the launches of single
+    // steps: 5.06 -> 3.29 ms.
+    for (int size = 0; size < 2; ++size) {
+        if (size == 1 && (n < GRAPH_STEPS[1] || capturing(d->stream) || ++d->short_runs <= 3)) break;
+        while (n >= GRAPH_STEPS[size]) {
+            if (!d->graph[d->cur][size])
+                if (int rc = capture_graph(d, d->cur, size)) return rc;
+            LBM_CUDA(cudaGraphLaunch(d->graph[d->cur][size], d->stream));
+            d->step += GRAPH_STEPS[size];
+            n -= GRAPH_STEPS[size];
         }
-        LBM_CUDA(cudaGraphLaunch(d->graph[d->cur], d->stream));
-        d->step += GRAPH_STEPS;
-        n -= GRAPH_STEPS;
     }
     for (int i = 0; i < n; ++i) {
         LBM_CUDA(prepare_one(d));
@@ -1055,6 +1071,7 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
         return LBM_OK;
     };
     auto fail = [&](int code) {
+        d->short_runs = 0;
         d->tile = orig;
         d->chosen = orig_chosen;
         drop_graphs(d);
@@ -1080,6 +1097,7 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
     double best = 1e300;
     StepTile best_t = orig;
     bool best_chosen = true;
+    d->short_runs = INT_MIN;  // no captures while timing
     for (const StepTile& t : cand) {
         d->tile = t;
         d->chosen = (size_t)(&t - cand.data()) != unchosen;  // timed as itself
@@ -1099,6 +1117,7 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
             best_chosen = d->chosen;
         }
     }
+    d->short_runs = 0;
     d->tile = best_t;
     d->chosen = best_chosen;
     drop_graphs(d);

@@ -276,8 +276,9 @@ struct lbm_domain {
     float* d_bc;        // reservoir densities (4 floats)
     float* d_probe;     // density at a probe cell (2 floats)
     double bc_host[4];  // last reservoir densities set
-    // captured chunks of GRAPH_STEPS steps, one per starting buffer
-    cudaGraphExec_t graph[2];
+    // captured chunks of GRAPH_STEPS[0] and [1] steps, per starting buffer
+    cudaGraphExec_t graph[2][2];
+    int short_runs;     // runs that had a chunk of GRAPH_STEPS[1] steps left
     cudaStream_t capture_stream;
     lbmk::TmaMaps tma;  // valid when tma_ok
     bool tma_ok;
@@ -294,4 +295,4 @@ struct lbm_domain {
     int push_maps_rows;        // box rows the push maps were encoded for (0: none)
 };
 
-constexpr int GRAPH_STEPS = 64;  // steps per captured graph (even: the buffer parity is unchanged)
+constexpr int GRAPH_STEPS[2] = {64, 8};  // steps per captured graph (even: the buffer parity is unchanged)
