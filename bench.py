@@ -496,13 +496,16 @@ def run_ours(args, rank, world, local):
 
     kind, _ = dom.step_kernel()
     h2 = "half2" if args.precision == 1 else "bfloat162"
-    # at tau = 1 two launches a step: an untuned domain, the two-launch kernel, and the
-    # 16-bit push kernel on boxes of 2^17 cells and more
-    two_launches = tuple(W.TAU) == (1.0, 1.0) and (
+    # two launches a step: an untuned domain and the two-launch kernel, and in 16-bit
+    # storage (at tau = 1 only) the push kernel on boxes of 2^17 cells and more
+    tau1 = tuple(W.TAU) == (1.0, 1.0)
+    two_launches = (tau1 or not args.precision) and (
         tuned is None or (kind == lbm.KERNEL_PUSH and box[0] * box[1] * box[2] >= 1 << 17 if args.precision
                           else kind == lbm.KERNEL_SPLIT))
     if two_launches and args.precision:
         kernel_name = "pair16_moment_kernel<%s> + pair16_push_kernel<%s> (one step)" % (h2, h2)
+    elif two_launches and not tau1:
+        kernel_name = "pair_moment_kernel + pair_relax_kernel (one step)"
     elif two_launches:
         kernel_name = ("moment_gather_kernel + moment_collide_kernel" if box[0] * box[1] * box[2] >= 5 << 17
                        else "pair_moment_kernel + pair_push_kernel") + " (one step)"
@@ -518,8 +521,6 @@ def run_ours(args, rank, world, local):
             rows, stages, ctas, "true" if tuple(W.TAU) == (1.0, 1.0) else "false", "true" if resident else "false")
     elif kind == lbm.KERNEL_TMA:
         kernel_name = "sc_step_tma_kernel"
-    elif kind == lbm.KERNEL_SPLIT:
-        kernel_name = "density_pair_kernel + sc_step_split_kernel (one step)"
     elif kind == lbm.KERNEL_STAGED2:
         kernel_name = "sc_step2_kernel<%d,2>" % lbm.lbm_get_tile(dom.h)[0]
     else:

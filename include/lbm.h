@@ -585,12 +585,12 @@ int lbm_get_tile(const lbm_domain* d, int* by, int* lz, int* lead);
  *                      32 x 8 tile with the tensor memory accelerator (boxes
  *                      without periodic x or y and with nx a multiple of 4);
  *                      lz planes per CTA z-segment (lz <= 0: the default);
- *   LBM_KERNEL_SPLIT   two launches per step: every cell's density pair into a
- *                      field, then pull + collision reading the 18 neighbour
- *                      densities from it (any box; FP32 only; lz ignored); with
- *                      tau = 1 in both components on the paired push layout
- *                      below, the second launch working from densities and
- *                      velocities alone, and on large boxes with the state kept
+ *   LBM_KERNEL_SPLIT   two launches per step on the paired push layout below:
+ *                      every cell's density pair into a field, then collision
+ *                      reading the 18 neighbour densities from it, and push (any
+ *                      box; FP32 only; lz ignored); with tau = 1 in both
+ *                      components the second launch works from densities and
+ *                      velocities alone, and on large boxes the state is kept
  *                      as each cell's densities, equilibrium velocities and rest
  *                      populations, from which its neighbours' populations are
  *                      formed (the staged kernel's results bit for bit);
@@ -624,8 +624,9 @@ int lbm_get_tile(const lbm_domain* d, int* by, int* lz, int* lead);
  *                      cells or more the same layout is stepped in two
  *                      launches, whatever the shape (the same bits).
  * New domains use LBM_KERNEL_STAGED; as long as neither a kernel nor a shape has
- * been chosen, a domain with tau = 1 in both components steps in two launches
- * (those of LBM_KERNEL_SPLIT, or their 16-bit counterpart), with the same bits
+ * been chosen, an FP32 domain, and a 16-bit domain with tau = 1 in both
+ * components, steps in two launches (those of LBM_KERNEL_SPLIT, or their 16-bit
+ * counterpart), with the same bits
  * (lbm_autotune times every kind that applies on the domain, and may leave a 16-bit
  * domain unchosen).  All give the same results up to rounding (not bit for bit:
  * the TMA kernel folds omega w_k into its equilibrium constants).  LBM_ERR_ARG

@@ -101,15 +101,17 @@ void drop_graphs(lbm_domain* d) {
     d->short_runs = std::min(d->short_runs, 0);  // counted anew; below 0: lbm_autotune is timing
 }
 
-// Whether steps run as the two launches of lbm_step_pairs.cu / lbm_step16_pairs.cu
-// (tau = 1 in both components): the two-launch kernel of FP32 domains, a domain that
-// nobody has chosen a kernel for -- the results are the staged kernel's bit for bit,
-// and on every box measured it is the faster one (a step of a 32^3 throat 10.4 -> 4.2
-// us, 48^3 periodic 16.1 -> 7.1 us, the 192^3 sample 0.69 -> 0.32 ms on moments) -- and
-// the push kernel of 16-bit domains from PAIRS16_CELLS cells on (same bits too).
+// Whether steps run as the two launches of lbm_step_pairs.cu / lbm_step16_pairs.cu (the
+// latter for tau = 1 in both components only): the two-launch kernel of FP32 domains, a
+// domain that nobody has chosen a kernel for -- the results are the staged kernel's bit
+// for bit, and on every box measured it is the faster one (tau = 1: a step of a 32^3
+// throat 10.4 -> 4.2 us, 48^3 periodic 16.1 -> 7.1 us, the 192^3 sample 0.69 -> 0.32 ms
+// on moments; tau = 0.8 and 1.2, periodic boxes: 16^3 8.7 -> 4.3 us, 48^3 16.2 -> 9.5,
+// 101 x 90 x 77 78 -> 48, 128^3 245 -> 147, 192^3 647 -> 507) -- and the push kernel of
+// 16-bit domains from PAIRS16_CELLS cells on (same bits too).
 constexpr long long PAIRS16_CELLS = 1LL << 17;  // 96^3: 75 -> 46 us a step, 192^3: 456 -> 433
 bool steps_in_pairs(const lbm_domain* d) {
-    if (!pair_step_applicable(d->phys)) return false;
+    if (d->params.precision != 0 && !pair_step_applicable(d->phys)) return false;
     if (d->tile.kind == LBM_KERNEL_STAGED) return !d->chosen;
     return d->params.precision == 0 ? d->tile.kind == LBM_KERNEL_SPLIT
                                     : d->tile.kind == LBM_KERNEL_PUSH && d->N >= PAIRS16_CELLS;
@@ -122,7 +124,7 @@ bool steps_in_pairs(const lbm_domain* d) {
 // 319 against 492.
 constexpr long long MOMENT_CELLS = 5LL << 17;
 bool steps_on_moments(const lbm_domain* d) {
-    return d->params.precision == 0 && steps_in_pairs(d) && d->N >= MOMENT_CELLS;
+    return d->params.precision == 0 && pair_step_applicable(d->phys) && steps_in_pairs(d) && d->N >= MOMENT_CELLS;
 }
 
 // One step from buffer `cur` to buffer cur ^ 1 (on moments: in place) on stream s.
@@ -148,9 +150,6 @@ cudaError_t launch_one(lbm_domain* d, int cur, cudaStream_t s) {
                                d->tile.tma_lz, d->d_err, s);
     if (d->params.precision == 0 && d->tile.kind == LBM_KERNEL_STAGED2)
         return launch_step2(d->f[cur], d->f[cur ^ 1], d->d_nbr, d->d_nbr_nw, d->d_adh, d->geom, d->phys, d->tile, s);
-    if (d->params.precision == 0 && d->tile.kind == LBM_KERNEL_SPLIT)
-        return launch_step_split(d->f[cur], d->f[cur ^ 1], d->d_rho2, d->d_nbr, d->d_nbr_nw, d->d_adh, d->geom,
-                                 d->phys, s);
     if (d->params.precision == 0)
         return launch_step(d->f[cur], d->f[cur ^ 1], d->d_nbr, d->d_nbr_nw, d->d_adh, d->geom, d->phys, d->tile, s);
     return launch_step16(d->params.precision, reinterpret_cast<const uint32_t*>(d->f[cur]),
@@ -164,7 +163,6 @@ cudaError_t prepare_one(lbm_domain* d) {
         return prepare_step16_push(d->params.precision, d->tile.push_shape);
     if (d->params.precision == 0 && d->tile.kind == LBM_KERNEL_PUSH) return prepare_step_push(d->tile.push_shape);
     if (d->params.precision == 0 && d->tile.kind == LBM_KERNEL_TMA) return prepare_step_tma();
-    if (d->params.precision == 0 && d->tile.kind == LBM_KERNEL_SPLIT) return cudaSuccess;
     if (d->params.precision == 0 && d->tile.kind == LBM_KERNEL_STAGED2) return prepare_step2(d->tile);
     return d->params.precision == 0 ? prepare_step(d->tile) : prepare_step16(d->params.precision, d->tile);
 }

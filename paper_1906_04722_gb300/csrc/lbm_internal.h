@@ -151,13 +151,9 @@ bool tile2_supported(int by, int lead);
 cudaError_t prepare_step2(const StepTile& t);
 cudaError_t launch_step2(const float* fin, float* fout, const uint32_t* nbr, const uint32_t* nbr_nw,
                          const uint32_t* adh, const Geom& g, const Phys& p, const StepTile& t, cudaStream_t s);
-// two-launch step: densities first, then pull + collide reading the neighbour
-// densities from rho2 (lbm_step_split.cu)
-cudaError_t launch_step_split(const float* fin, float* fout, float2* rho2, const uint32_t* nbr,
-                              const uint32_t* nbr_nw, const uint32_t* adh, const Geom& g, const Phys& p,
-                              cudaStream_t s);
-// the same for tau = 1 in both components, on the paired push layout; fin is left
-// with the step's intermediate values (lbm_step_pairs.cu)
+// two-launch step on the paired push layout; at tau = 1 in both components
+// (pair_step_applicable) fin is left with the step's intermediate values
+// (lbm_step_pairs.cu)
 bool pair_step_applicable(const Phys& p);
 cudaError_t launch_step_pairs(float* fin, float* fout, float2* rho2, const uint32_t* nbr, const uint32_t* nbr_nw,
                               const uint32_t* adh, const Geom& g, const Phys& p, cudaStream_t s);

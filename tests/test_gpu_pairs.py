@@ -1,8 +1,8 @@
-"""The two-launch step at tau = 1 (LBM_KERNEL_SPLIT, and the route of a domain
-without a chosen kernel) against the staged kernel, bit for bit: ragged and odd
-boxes, every periodic axis, boxes one or two cells wide, membrane and reservoirs,
-body force, boxes large enough to step on moments; switching kernels on the way;
-unequal tau keeps the other two-launch kernel.
+"""The two-launch step (LBM_KERNEL_SPLIT, and the route of a domain without a
+chosen kernel) against the staged kernel, bit for bit: ragged and odd boxes, every
+periodic axis, boxes one or two cells wide, membrane and reservoirs, body force,
+boxes large enough to step on moments; switching kernels on the way; at tau = 1 and
+at others.
 """
 import numpy as np
 import pytest
@@ -98,6 +98,28 @@ def test_unequal_tau(lbm):
     c.set_step_kernel(lbm.KERNEL_SPLIT)
     c.step(20)
     assert np.allclose(c.density(), a.density(), rtol=1e-5, atol=1e-7)
+
+
+@pytest.mark.parametrize("tau", [(0.8, 1.2), (1.0, 1.2), (0.7, 0.7)])
+@pytest.mark.parametrize("shape,periodic,par", [
+    ((29, 21, 37), (0, 0, 0), {}),
+    ((31, 20, 34), (0, 1, 1), {"body_force": (1e-5, -2e-5, 3e-5)}),
+    ((40, 22, 35), (0, 0, 0), {"reservoirs": True, "membrane_layers": 3}),
+    ((9, 1, 40), (0, 1, 0), {}),
+    ((2, 19, 2), (1, 1, 1), {}),
+    ((90, 87, 89), (0, 0, 1), {}),
+])
+def test_any_tau_equals_the_staged_kernel(lbm, shape, periodic, par, tau):
+    staged = _domain(lbm, shape, periodic, tau=tau, **par)
+    staged.set_step_kernel(lbm.KERNEL_STAGED)
+    want = _read(staged, 70)
+    _equal(_read(_domain(lbm, shape, periodic, tau=tau, **par), 70), want)
+    d = _domain(lbm, shape, periodic, tau=tau, **par)
+    d.step(13)
+    d.set_step_kernel(lbm.KERNEL_STAGED)
+    d.step(30)
+    d.set_step_kernel(lbm.KERNEL_SPLIT)
+    _equal(_read(d, 27), want)
 
 
 @pytest.mark.parametrize("precision", [1, 2])
