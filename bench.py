@@ -342,9 +342,9 @@ def throat_bench(lbm, W, n_steps, rank, world, sync, tmax, gather=None):
         rel = np.abs(est[ok] - truth[ok]) / np.abs(truth[ok])
         out["baselines"][name] = {"median_ratio_to_lbm": float(np.median(est[ok] / truth[ok])),
                                   "rel_err_median": float(np.median(rel)), "rel_err_p90": float(np.percentile(rel, 90))}
-    out["batch_form"] = ("cell list: compact storage of every non-solid cell, a density launch and a push-streaming "
-                         "step launch per time step")
-    # the same batch in the other two forms, for context
+    out["batch_form"] = ("on chip: a throat's non-solid cells in the shared memory of one thread-block cluster for all "
+                         "steps of an increment (tau = 1; throats that do not fit: the cell list)")
+    # the same batch in other forms, for context
     out["other_forms"] = {}
     agree = True
     for form, name in ((lbm.BATCH_MARCH, "march"), (lbm.BATCH_PER_STEP, "tiles_per_step"),

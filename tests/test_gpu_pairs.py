@@ -155,3 +155,19 @@ def test_16_bit(lbm, precision, shape, periodic, par):
         a, b = d.measure(allow_nonfinite=True), staged.measure(allow_nonfinite=True)
         assert a["n_w"] == b["n_w"] and a["n_interface"] == b["n_interface"]
         assert d.density_at(1, 5, 1) == staged.density_at(1, 5, 1)
+
+
+@pytest.mark.parametrize("precision,par,shape", [
+    (0, {}, (29, 21, 37)), (1, {}, (29, 21, 37)), (0, {"tau": (0.8, 1.2)}, (29, 21, 37)), (0, {}, (90, 87, 89)),
+])
+def test_short_runs_equal_one_long_run(lbm, precision, par, shape):
+    runs = [7, 8, 25, 9, 31, 8, 63, 25]  # chunks of 8 replay a graph from the fourth run of 8 and more on
+    a = _domain(lbm, shape, (0, 0, 1), precision=precision, **par)
+    b = _domain(lbm, shape, (0, 0, 1), precision=precision, **par)
+    b.set_step_kernel(lbm.KERNEL_STAGED)
+    b.step(sum(runs) + 2 * 20)
+    for n in runs:
+        a.step(n)
+    a.set_step_kernel(lbm.KERNEL_STAGED)  # drops the graphs
+    a.step(20)
+    _equal(_read(a, 20), _read(b, 0))
