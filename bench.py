@@ -496,12 +496,10 @@ def run_ours(args, rank, world, local):
 
     kind, _ = dom.step_kernel()
     h2 = "half2" if args.precision == 1 else "bfloat162"
-    # two launches a step: an untuned domain and the two-launch kernel, and in 16-bit
-    # storage (at tau = 1 only) the push kernel on boxes of 2^17 cells and more
+    # two launches a step: the two-launch kernel, and an untuned domain (in 16-bit storage
+    # at tau = 1 only)
     tau1 = tuple(W.TAU) == (1.0, 1.0)
-    two_launches = (tau1 or not args.precision) and (
-        tuned is None or (kind == lbm.KERNEL_PUSH and box[0] * box[1] * box[2] >= 1 << 17 if args.precision
-                          else kind == lbm.KERNEL_SPLIT))
+    two_launches = kind == lbm.KERNEL_SPLIT or (tuned is None and (tau1 or not args.precision))
     if two_launches and args.precision:
         kernel_name = "pair16_moment_kernel<%s> + pair16_push_kernel<%s> (one step)" % (h2, h2)
     elif two_launches and not tau1:
@@ -600,7 +598,7 @@ def run_ours(args, rank, world, local):
            "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                         "frac": achieved / peak, "traffic": read_traffic(kernel_name) if args.size == 192 else None, "peak_kind": peak_kind,
                         "kernel": kernel_name, "algorithmic_bytes_per_launch": bytes_per_step},
-           "gpu_launches": args.steps * (2 if two_launches or (kind == lbm.KERNEL_SPLIT and not args.precision) else 1),
+           "gpu_launches": args.steps * (2 if two_launches else 1),
            "e2e": {"value": e2e_val, "unit": "MLUPS", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                    "step": f"set_pressure_bc + {E2E_SUBSTEPS} time steps + lbm_measure; domain creation "
                            "from the host sphere list inside the timed region"},

@@ -576,8 +576,8 @@ int lbm_measure_state_noalloc(const lbm_params* params, const int box[3], const 
 int lbm_set_tile(lbm_domain* d, int by, int lz, int lead);
 int lbm_get_tile(const lbm_domain* d, int* by, int* lz, int* lead);
 
-/* lbm_set_step_kernel / lbm_get_step_kernel -- which kernel advances an FP32
- * domain (16-bit storage always uses the staged kernel).
+/* lbm_set_step_kernel / lbm_get_step_kernel -- which kernel advances a domain
+ * (16-bit storage: STAGED, PUSH and, with tau = 1 in both components, SPLIT).
  *   LBM_KERNEL_STAGED  every thread queues its cell's 2 x 19 pulls as 4-byte
  *                      asynchronous copies (any box, any periodic axes); its
  *                      shape is set with lbm_set_tile;
@@ -588,7 +588,8 @@ int lbm_get_tile(const lbm_domain* d, int* by, int* lz, int* lead);
  *   LBM_KERNEL_SPLIT   two launches per step on the paired push layout below:
  *                      every cell's density pair into a field, then collision
  *                      reading the 18 neighbour densities from it, and push (any
- *                      box; FP32 only; lz ignored); with tau = 1 in both
+ *                      box; lz ignored; 16-bit storage: on its push layout, with
+ *                      tau = 1 in both components only); with tau = 1 in both
  *                      components the second launch works from densities and
  *                      velocities alone, and on large boxes the state is kept
  *                      as each cell's densities, equilibrium velocities and rest
@@ -620,15 +621,11 @@ int lbm_get_tile(const lbm_domain* d, int* by, int* lz, int* lead);
  *                      density pairs per plane (boxes without periodic x or y
  *                      and with nx % 4 == 0).  Its results equal the staged
  *                      16-bit kernel's bit for bit; the read-outs read
- *                      either layout.  With tau = 1 in both components and 2^17
- *                      cells or more the same layout is stepped in two
- *                      launches, whatever the shape (the same bits).
+ *                      either layout.
  * New domains use LBM_KERNEL_STAGED; as long as neither a kernel nor a shape has
  * been chosen, an FP32 domain, and a 16-bit domain with tau = 1 in both
- * components, steps in two launches (those of LBM_KERNEL_SPLIT, or their 16-bit
- * counterpart), with the same bits
- * (lbm_autotune times every kind that applies on the domain, and may leave a 16-bit
- * domain unchosen).  All give the same results up to rounding (not bit for bit:
+ * components, steps in the two launches of LBM_KERNEL_SPLIT, with the same bits
+ * (lbm_autotune times every kind that applies on the domain).  All give the same results up to rounding (not bit for bit:
  * the TMA kernel folds omega w_k into its equilibrium constants).  LBM_ERR_ARG
  * for an unknown kind, LBM_ERR_STATE when the kernel does not apply to the
  * domain.  lbm_set_tile switches the domain to LBM_KERNEL_STAGED. */
@@ -700,8 +697,10 @@ int lbm_set_push_order(lbm_domain* d, int order);
  * staged kernel (by 6 or 8, z segments of 8 .. 32), and the staged kernel with
  * by in {6, 8, 10}, lead in {0, 1, 2, 3} (0 and 1: the double-pull variant) and
  * z segments of 8 .. 32 planes; for 16-bit storage the staged kernel with by in
- * {6, 8, 10} and lead 2 and (where it applies) the 16-bit push kernel in every
- * shape with z segments of 16, 24, 32 and 48 planes.
+ * {6, 8, 10} and lead 2, (where it applies) the 16-bit push kernel in every
+ * shape with z segments of 16, 24, 32 and 48 planes and (tau = 1 in both
+ * components) the two-launch kernel.  Each candidate is a kernel and shape that
+ * the calls above set: they take another domain to what was timed here.
  * Timing uses CUDA events on the domain's stream.  The
  * populations, the step counter and (16-bit) the density fields are saved
  * before and restored after, bit for bit: a tuned domain continues exactly where

@@ -102,19 +102,15 @@ void drop_graphs(lbm_domain* d) {
 }
 
 // Whether steps run as the two launches of lbm_step_pairs.cu / lbm_step16_pairs.cu (the
-// latter for tau = 1 in both components only): the two-launch kernel of FP32 domains, a
-// domain that nobody has chosen a kernel for -- the results are the staged kernel's bit
-// for bit, and on every box measured it is the faster one (tau = 1: a step of a 32^3
-// throat 10.4 -> 4.2 us, 48^3 periodic 16.1 -> 7.1 us, the 192^3 sample 0.69 -> 0.32 ms
-// on moments; tau = 0.8 and 1.2, periodic boxes: 16^3 8.7 -> 4.3 us, 48^3 16.2 -> 9.5,
-// 101 x 90 x 77 78 -> 48, 128^3 245 -> 147, 192^3 647 -> 507) -- and the push kernel of
-// 16-bit domains from PAIRS16_CELLS cells on (same bits too).
-constexpr long long PAIRS16_CELLS = 1LL << 17;  // 96^3: 75 -> 46 us a step, 192^3: 456 -> 433
+// latter for tau = 1 in both components only): the two-launch kernel, and a domain that
+// nobody has chosen a kernel for -- the results are the staged kernel's bit for bit, and
+// on every box measured it is the faster one (tau = 1: a step of a 32^3 throat 10.4 ->
+// 4.2 us, 48^3 periodic 16.1 -> 7.1 us, the 192^3 sample 0.69 -> 0.32 ms on moments;
+// tau = 0.8 and 1.2, periodic boxes: 16^3 8.7 -> 4.3 us, 48^3 16.2 -> 9.5, 101 x 90 x 77
+// 78 -> 48, 128^3 245 -> 147, 192^3 647 -> 507; 16-bit: 32^3 throat 9.4 -> 4.7 us).
 bool steps_in_pairs(const lbm_domain* d) {
     if (d->params.precision != 0 && !pair_step_applicable(d->phys)) return false;
-    if (d->tile.kind == LBM_KERNEL_STAGED) return !d->chosen;
-    return d->params.precision == 0 ? d->tile.kind == LBM_KERNEL_SPLIT
-                                    : d->tile.kind == LBM_KERNEL_PUSH && d->N >= PAIRS16_CELLS;
+    return d->tile.kind == LBM_KERNEL_SPLIT || (d->tile.kind == LBM_KERNEL_STAGED && !d->chosen);
 }
 
 // Whether such a domain's steps run on moments (lbm_step_moments.cu), in place in one
@@ -897,8 +893,12 @@ int lbm_set_step_kernel(lbm_domain* d, int kind, int lz) {
         drop_graphs(d);
         return fp32 ? ensure_push_maps(d) : ensure_push16_maps(d);
     }
-    if ((kind == LBM_KERNEL_SPLIT || kind == LBM_KERNEL_STAGED2) && d->params.precision != 0) {
-        set_error("the two-launch and two-threads-per-cell step kernels need an FP32 domain");
+    if (kind == LBM_KERNEL_STAGED2 && d->params.precision != 0) {
+        set_error("the two-threads-per-cell step kernel needs an FP32 domain");
+        return LBM_ERR_STATE;
+    }
+    if (kind == LBM_KERNEL_SPLIT && d->params.precision != 0 && !pair_step_applicable(d->phys)) {
+        set_error("the two-launch step kernel needs an FP32 domain, or tau = 1 in both components");
         return LBM_ERR_STATE;
     }
     if (kind == LBM_KERNEL_STAGED2) {
@@ -994,7 +994,6 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
     const int layout = d->layout;
     // candidates
     std::vector<StepTile> cand;
-    size_t unchosen = SIZE_MAX;  // the candidate that stands for the route of a domain without a chosen kernel
     auto add = [&](int kind, int by, int lz, int lead) {
         StepTile t = orig;
         t.kind = kind;
@@ -1029,18 +1028,9 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
                 t.push_order = 0;
                 cand.push_back(t);
             }
-    if (!fp32 && pair_step_applicable(d->phys)) {  // reachable in no other way on a small 16-bit box
-        unchosen = cand.size();
-        StepTile t = default_tile(g);
-        t.push_shape = orig.push_shape;
-        t.push_lz = orig.push_lz;
-        t.push_pf = orig.push_pf;
-        t.push_order = orig.push_order;
-        cand.push_back(t);
-    }
     if (fp32 && d->tma_ok)
         for (int lz : {8, 12, 16, 24, 32, 48}) add(LBM_KERNEL_TMA, orig.by, lz, orig.lead);
-    if (fp32) add(LBM_KERNEL_SPLIT, orig.by, orig.lz, orig.lead);
+    if (fp32 || pair_step_applicable(d->phys)) add(LBM_KERNEL_SPLIT, orig.by, orig.lz, orig.lead);
     if (fp32)
         for (int by : {6, 8})
             for (int lz : {8, 16, 32}) add(LBM_KERNEL_STAGED2, by, lz, 2);
@@ -1094,11 +1084,10 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
     }
     double best = 1e300;
     StepTile best_t = orig;
-    bool best_chosen = true;
     d->short_runs = INT_MIN;  // no captures while timing
+    d->chosen = true;
     for (const StepTile& t : cand) {
         d->tile = t;
-        d->chosen = (size_t)(&t - cand.data()) != unchosen;  // timed as itself
         drop_graphs(d);
         if ((rc = restore())) return fail(rc);
         if ((rc = run_steps(d, 1))) return fail(rc);  // untimed: kernel set-up, ghost stores
@@ -1112,12 +1101,10 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
         if (per < best) {
             best = per;
             best_t = t;
-            best_chosen = d->chosen;
         }
     }
     d->short_runs = 0;
     d->tile = best_t;
-    d->chosen = best_chosen;
     drop_graphs(d);
     if ((rc = restore())) return fail(rc);
     if (d->layout == 0)
