@@ -129,7 +129,13 @@ int lbm_set_pressure_bc(lbm_domain* d, double rho_in_nw, double rho_out_w);
  * captured on first use (one per starting buffer, recaptured after
  * lbm_set_tile), chunks of 8 another one once the domain has been stepped in short
  * runs a few times; the remainder is launched step by step.  Results are the same
- * either way, bit for bit. */
+ * either way, bit for bit.
+ * A caller may capture an even number of steps on the domain's stream and replay
+ * them, after lbm_set_densities or lbm_set_state too (the step counter counts the
+ * captured steps once).  From then on a domain that LBM_KERNEL_SPLIT advances, or no
+ * chosen kernel, steps with the staged kernel: the same bits, on the layout that a
+ * state is set in.  With LBM_KERNEL_PUSH, whose state is kept in another layout, take
+ * a step before the capture, and capture anew after the state has been set. */
 int lbm_step(lbm_domain* d, int n_steps);
 
 /* lbm_measure -- observables of the current state (synchronises the domain's

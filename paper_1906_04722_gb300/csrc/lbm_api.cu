@@ -109,7 +109,7 @@ void drop_graphs(lbm_domain* d) {
 // tau = 0.8 and 1.2, periodic boxes: 16^3 8.7 -> 4.3 us, 48^3 16.2 -> 9.5, 101 x 90 x 77
 // 78 -> 48, 128^3 245 -> 147, 192^3 647 -> 507; 16-bit: 32^3 throat 9.4 -> 4.7 us).
 bool steps_in_pairs(const lbm_domain* d) {
-    if (d->params.precision != 0 && !pair_step_applicable(d->phys)) return false;
+    if (d->pull_steps || (d->params.precision != 0 && !pair_step_applicable(d->phys))) return false;
     return d->tile.kind == LBM_KERNEL_SPLIT || (d->tile.kind == LBM_KERNEL_STAGED && !d->chosen);
 }
 
@@ -287,16 +287,53 @@ int capture_graph(lbm_domain* d, int parity, int size) {
     return LBM_OK;
 }
 
-bool capturing(cudaStream_t s) {
+// Whether a caller may capture the domain's stream, and whether one does now.
+bool capturable(const lbm_domain* d) { return d->stream && d->stream != cudaStreamLegacy; }
+bool capturing(const lbm_domain* d) {
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
-    cudaGetLastError();  // the legacy stream while another stream captures
-    return true;
+    if (capturable(d) && cudaStreamIsCapturing(d->stream, &st) != cudaSuccess) cudaGetLastError();
+    return st != cudaStreamCaptureStatusNone;
+}
+
+// Steps captured by a caller are replayed any number of times, and after the state has
+// been set anew: they have to start and end in the layout that a state is set in.  From
+// its first captured steps on, a domain of the two-launch kernel therefore stays on the
+// pull layout, with the staged kernel (the same bits).  The conversion of a state that is
+// in another layout is no part of the graph: it runs at once, on the private stream,
+// behind the steps that were queued before the capture.
+int keep_pull(lbm_domain* d) {
+    if (d->layout != 0) {
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;  // for this thread, while it waits
+        LBM_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+        auto convert = [&]() -> int {
+            if (!d->capture_stream) LBM_CUDA(cudaStreamCreateWithFlags(&d->capture_stream, cudaStreamNonBlocking));
+            LBM_CUDA(cudaStreamWaitEvent(d->capture_stream, d->stepped, 0));
+            const cudaStream_t stream = d->stream;
+            d->stream = d->capture_stream;
+            const int rc = set_layout(d, 0);
+            d->stream = stream;
+            if (rc) return rc;
+            LBM_CUDA(cudaStreamSynchronize(d->capture_stream));
+            return LBM_OK;
+        };
+        const int rc = convert();
+        LBM_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+        if (rc) return rc;
+    }
+    d->pull_steps = true;
+    return LBM_OK;
 }
 
 // n steps: whole chunks replay captured graphs, the remainder is launched one by one.
 int run_steps(lbm_domain* d, int n) {
     if (n <= 0) return LBM_OK;
+    const bool captured = capturing(d);
+    if (captured && steps_in_pairs(d))
+        if (int rc = keep_pull(d)) return rc;
+    if (!captured && d->graphs_pull != d->pull_steps) {
+        drop_graphs(d);
+        d->graphs_pull = d->pull_steps;
+    }
     const bool moments = steps_on_moments(d);
     if (!moments || d->layout != 2)
         if (int rc = set_layout(d, wanted_layout(d))) return rc;
@@ -324,8 +361,8 @@ int run_steps(lbm_domain* d, int n) {
     // or three such runs); not while a caller captures the domain's stream.  A 32^3
     // throat's ladder of 20 x 25 two-launch steps is bound by the launches of single
     // steps: 5.06 -> 3.29 ms.
-    for (int size = 0; size < 2; ++size) {
-        if (size == 1 && (n < GRAPH_STEPS[1] || capturing(d->stream) || ++d->short_runs <= 3)) break;
+    for (int size = 0; size < 2 && !captured; ++size) {
+        if (size == 1 && (n < GRAPH_STEPS[1] || ++d->short_runs <= 3)) break;
         while (n >= GRAPH_STEPS[size]) {
             if (!d->graph[d->cur][size])
                 if (int rc = capture_graph(d, d->cur, size)) return rc;
@@ -340,6 +377,7 @@ int run_steps(lbm_domain* d, int n) {
         if (!moments) d->cur ^= 1;
         ++d->step;
     }
+    if (!captured && d->layout != 0 && capturable(d)) LBM_CUDA(cudaEventRecord(d->stepped, d->stream));
     return LBM_OK;
 }
 
@@ -366,6 +404,7 @@ void free_domain(lbm_domain* d) {
     if (d->capture_stream) cudaStreamDestroy(d->capture_stream);
     if (d->h_result) cudaFreeHost(d->h_result);
     if (d->done) cudaEventDestroy(d->done);
+    if (d->stepped) cudaEventDestroy(d->stepped);
     delete d;
 }
 
@@ -432,14 +471,15 @@ __global__ void to_double_kernel(const float* __restrict__ in, double* __restric
 
 // Build the stored populations from the densities in d->d_rho.
 int init_from_densities(lbm_domain* d) {
+    const int cur = d->pull_steps ? d->cur : 0;  // a caller's graph starts from the buffer that is current
     if (d->params.precision == 0) {
-        LBM_CUDA(launch_init(d->d_rho, d->f[0], d->d_nbr, d->d_nbr_nw, d->geom, d->stream));
+        LBM_CUDA(launch_init(d->d_rho, d->f[cur], d->d_nbr, d->d_nbr_nw, d->geom, d->stream));
     } else {
-        LBM_CUDA(cudaMemsetAsync(d->f[0], 0, sizeof(uint32_t) * (size_t)d->geom.plane * Q, d->stream));
-        LBM_CUDA(launch_init16(d->d_rho, d->R[0], d->geom, d->stream));
+        LBM_CUDA(cudaMemsetAsync(d->f[cur], 0, sizeof(uint32_t) * (size_t)d->geom.plane * Q, d->stream));
+        LBM_CUDA(launch_init16(d->d_rho, d->R[cur], d->geom, d->stream));
     }
     const bool dirty = d->layout != 0;
-    d->cur = 0;
+    d->cur = cur;
     d->step = 0;
     d->ghosts_ok = false;
     d->layout = 0;
@@ -574,6 +614,7 @@ int create_common(const lbm_params* params, const uint8_t* mask_host, const int 
     // FP32: 2 x 19 floats per cell; 16-bit: 19 pair words per cell plus the density pair
     const size_t fbytes = (params->precision == 0 ? sizeof(float) * 2 : sizeof(uint32_t)) * (size_t)g.plane * Q;
     LBM_CUDA_D(cudaEventCreateWithFlags(&d->done, cudaEventDisableTiming));
+    LBM_CUDA_D(cudaEventCreateWithFlags(&d->stepped, cudaEventDisableTiming));
     LBM_CUDA_D(cudaMalloc(&d->f[0], fbytes));
     LBM_CUDA_D(cudaMalloc(&d->f[1], fbytes));
     if (params->precision != 0) {
@@ -1030,7 +1071,7 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
             }
     if (fp32 && d->tma_ok)
         for (int lz : {8, 12, 16, 24, 32, 48}) add(LBM_KERNEL_TMA, orig.by, lz, orig.lead);
-    if (fp32 || pair_step_applicable(d->phys)) add(LBM_KERNEL_SPLIT, orig.by, orig.lz, orig.lead);
+    if (!d->pull_steps && (fp32 || pair_step_applicable(d->phys))) add(LBM_KERNEL_SPLIT, orig.by, orig.lz, orig.lead);
     if (fp32)
         for (int by : {6, 8})
             for (int lz : {8, 16, 32}) add(LBM_KERNEL_STAGED2, by, lz, 2);

@@ -274,6 +274,9 @@ struct lbm_domain {
     double bc_host[4];  // last reservoir densities set
     // captured chunks of GRAPH_STEPS[0] and [1] steps, per starting buffer
     cudaGraphExec_t graph[2][2];
+    bool pull_steps;    // a caller's graph holds steps of this domain: it stays on the pull layout (keep_pull)
+    bool graphs_pull;   // pull_steps when the chunks' graphs were captured
+    cudaEvent_t stepped;  // behind the last steps queued on a stream that may be captured
     int short_runs;     // runs that had a chunk of GRAPH_STEPS[1] steps left
     cudaStream_t capture_stream;
     lbmk::TmaMaps tma;  // valid when tma_ok
