@@ -1090,7 +1090,7 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
         if (e0) cudaEventDestroy(e0);
         if (e1) cudaEventDestroy(e1);
     };
-    auto restore = [&]() -> int {
+    auto rewind = [&]() -> int {
         LBM_CUDA(cudaMemcpyAsync(d->f[cur], fsave, fbytes, cudaMemcpyDeviceToDevice, d->stream));
         if (rbytes) LBM_CUDA(cudaMemcpyAsync(d->R[cur], rsave, rbytes, cudaMemcpyDeviceToDevice, d->stream));
         d->cur = cur;
@@ -1098,6 +1098,11 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
         d->layout = layout;
         d->ghosts_ok = false;
         return LBM_OK;
+    };
+    // for good: what the candidates left in the other buffer goes too
+    auto restore = [&]() -> int {
+        if (int r = rewind()) return r;
+        return d->layout == 0 ? clear_other(d) : LBM_OK;
     };
     auto fail = [&](int code) {
         d->short_runs = 0;
@@ -1130,7 +1135,7 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
     for (const StepTile& t : cand) {
         d->tile = t;
         drop_graphs(d);
-        if ((rc = restore())) return fail(rc);
+        if ((rc = rewind())) return fail(rc);
         if ((rc = run_steps(d, 1))) return fail(rc);  // untimed: kernel set-up, ghost stores
         if (cudaEventRecord(e0, d->stream) != cudaSuccess) return fail(LBM_ERR_CUDA);
         if ((rc = run_steps(d, trial_steps))) return fail(rc);
@@ -1148,8 +1153,6 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
     d->tile = best_t;
     drop_graphs(d);
     if ((rc = restore())) return fail(rc);
-    if (d->layout == 0)
-        if ((rc = clear_other(d))) return fail(rc);
     rc = wait_domain(d);
     cleanup();
     if (rc) return rc;
