@@ -1083,6 +1083,7 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
             }
     void* fsave = nullptr;
     void* rsave = nullptr;
+    bool saved = false;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     auto cleanup = [&]() {
         cudaFree(fsave);
@@ -1109,7 +1110,7 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
         d->tile = orig;
         d->chosen = orig_chosen;
         drop_graphs(d);
-        if (fsave) restore();
+        if (saved) restore();
         wait_domain(d);
         cleanup();
         return code;
@@ -1128,6 +1129,7 @@ int lbm_autotune(lbm_domain* d, int trial_steps, lbm_tune_result* out) {
         set_error(std::string("lbm_autotune: ") + cudaGetErrorString(e));
         return fail(LBM_ERR_CUDA);
     }
+    saved = true;
     double best = 1e300;
     StepTile best_t = orig;
     d->short_runs = INT_MIN;  // no captures while timing
