@@ -527,7 +527,8 @@ lbm_surrogate* lbm_throat_surrogate_network(lbm_throat_surrogate* ts);
 void lbm_throat_surrogate_destroy(lbm_throat_surrogate* ts);
 
 /* lbm_get_density -- densities of the current state, 2 x N doubles
- * (component-major), 0 where a component is not fluid. Synchronising. */
+ * (component-major), 0 where a component is not fluid. Synchronising.  rho_out is
+ * written (as lbm_get_state's f_out is) once the work queued so far has succeeded. */
 int lbm_get_density(lbm_domain* d, double* rho_out);
 
 /* lbm_get_mask -- the domain's mask, N bytes. */

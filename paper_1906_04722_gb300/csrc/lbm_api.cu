@@ -838,12 +838,18 @@ int lbm_get_density(lbm_domain* d, double* rho_out) {
                                       d->R[d->cur], d->d_nbr, d->d_nbr_nw, d->geom, d->layout == 1, d->d_rho,
                                       d->stream));
         }
-        touch_pages(rho_out, sizeof(double) * 2 * (size_t)d->N);
-        for (long long i = 0; i < 2 * d->N; i += CONVERT_PIECE) {
-            const long long n = std::min(CONVERT_PIECE, 2 * d->N - i);
-            to_double_kernel<<<1216, 256, 0, d->stream>>>(d->d_rho + i, d->d_convert, n);
-            LBM_CUDA(cudaGetLastError());
-            LBM_CUDA(cudaMemcpyAsync(rho_out + i, d->d_convert, sizeof(double) * n, cudaMemcpyDeviceToHost, d->stream));
+        const long long total = 2 * d->N;
+        auto convert = [&](long long i) {  // the piece from value i on
+            to_double_kernel<<<1216, 256, 0, d->stream>>>(d->d_rho + i, d->d_convert, std::min(CONVERT_PIECE, total - i));
+            return cudaGetLastError();
+        };
+        LBM_CUDA(convert(0));
+        if (int rc = wait_domain(d)) return rc;  // nothing is written before the device work has succeeded
+        touch_pages(rho_out, sizeof(double) * (size_t)total);
+        for (long long i = 0; i < total; i += CONVERT_PIECE) {
+            if (i) LBM_CUDA(convert(i));
+            LBM_CUDA(cudaMemcpyAsync(rho_out + i, d->d_convert, sizeof(double) * std::min(CONVERT_PIECE, total - i),
+                                     cudaMemcpyDeviceToHost, d->stream));
         }
         return wait_domain(d);
     } catch (const std::bad_alloc&) {
@@ -873,6 +879,7 @@ int lbm_get_state(lbm_domain* d, float* f_out, long long* step_out) {
     const long long N = d->N;
     const float* fp = nullptr;
     if (int rc = pull_view(d, &fp)) return rc;
+    if (int rc = wait_domain(d)) return rc;  // nothing is written before the device work has succeeded
     touch_pages(f_out, sizeof(float) * 2 * Q * (size_t)N);
     for (int p = 0; p < 2 * Q; ++p)
         LBM_CUDA(cudaMemcpyAsync(f_out + (size_t)p * N, fp + (size_t)p * d->geom.plane, sizeof(float) * N,

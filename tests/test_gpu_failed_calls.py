@@ -58,10 +58,10 @@ def _in_thread(call):
     return t, got
 
 
-def _domain(lbm):
+def _domain(lbm, precision=0):
     import torch
     nz, ny, nx = SHAPE
-    p = lbm.make_params(rho_major=W.RHO_MAJOR, rho_minor=W.RHO_MINOR)
+    p = lbm.make_params(rho_major=W.RHO_MAJOR, rho_minor=W.RHO_MINOR, precision=precision)
     d = lbm.Domain(p, SPHERES, (nx, ny, nz), stream=torch.cuda.Stream().cuda_stream)
     d.set_densities(W.droplet_densities(SHAPE, (nx / 2, ny / 2, nz / 2), 20.0, seed=5))
     return d
@@ -86,3 +86,31 @@ def test_a_failed_autotune_leaves_the_domain_as_it_was(lbm):
         ref.step(n)
         a, b = d.state(), ref.state()
         assert np.array_equal(a[0], b[0]) and a[1] == b[1]
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("call", ["density", "state"])
+def test_a_failed_read_out_leaves_the_array_as_it_was(lbm, call, precision):
+    if call == "state" and precision:
+        pytest.skip("16-bit domains have no checkpoints")
+    d = _domain(lbm, precision)
+    d.step(3)
+    n = int(np.prod(SHAPE)) * (2 if call == "density" else 38)
+    out = np.full(n, 7.0, np.float64 if call == "density" else np.float32)
+    L = lbm.load()
+    if call == "density":
+        def read():
+            return L.lbm_get_density(d.h, out.ctypes.data_as(ctypes.POINTER(ctypes.c_double)))
+    else:
+        step = ctypes.c_longlong(0)
+
+        def read():
+            return L.lbm_get_state(d.h, out.ctypes.data_as(ctypes.POINTER(ctypes.c_float)), ctypes.byref(step))
+    with _waits_refused():
+        t, got = _in_thread(read)
+        t.join()
+    assert got[0] != 0
+    assert np.all(out == 7.0)
+    assert read() == 0
+    want = d.density() if call == "density" else d.state()[0]
+    assert np.array_equal(out, want.ravel())
