@@ -5,13 +5,14 @@ Workload (default): the fully resolved drainage sample, 192^3 lattice, 300
 non-overlapping spheres with radii U[10, 14] placed by seeded random
 sequential addition, inlet reservoir layer z = 0, three membrane layers and
 the outlet reservoir layer at the top, FP32 populations.  One bench step is
-one time step of the whole domain (one launch of the fused step kernel).
+one time step of the whole domain (one launch, or two: config.workload says).
 
 Printed JSON line (rank 0):
   value      fluid-cell updates per second (MLUPS) with the state resident in
              HBM, CUDA events around exactly --steps launches, max over ranks;
-  roofline   the step kernel against HBM bandwidth: algorithmic bytes
-             (2 x 19 populations read + written per fluid cell) / mean launch time;
+  roofline   the step against HBM bandwidth: the bytes that the kernel in use has
+             to move / mean step time, and beside it (populations) the same with
+             2 x 19 populations read + written per fluid cell;
   e2e        the same metric through the public C ABI from host data: domain
              creation from the host sphere list, then per step
              set_pressure_bc + 100 time steps + a measurement read back;
@@ -19,7 +20,7 @@ Printed JSON line (rank 0):
   throats    pore throats per second on 1024 Delaunay throats of the sample
              packing (boxes 24^3..64^3): the plain per-throat loop (create,
              ladder of set_pressure_bc + steps + measure, destroy) on a strided
-             subset, the batch (cell-list form, with the tile and persistent
+             subset, the batch (on chip, with the marching, tile and persistent
              forms beside it), and the surrogate (trained on six other packings)
              with batched-LBM fallback where the ensemble spread exceeds 2 % (and
              5 %), with the surrogate's p_c^e error against the batched LBM.
@@ -163,13 +164,35 @@ KERNEL_SOURCES = {
     "sc_step16_push_kernel": ("lbm_step16_push.cuh", "lbm_step16_push.cu", "lbm_step16_push_bf16.cu",
                               "lbm_pair16.cuh", "lbm_push_tma.cuh", "lbm_step_core.cuh", "lbm_device.cuh",
                               "lbm_internal.h"),
+    "moment_gather_kernel": ("lbm_step_moments.cu", "lbm_collide_pair.cuh", "lbm_device.cuh", "lbm_internal.h"),
+    "pair_moment_kernel": ("lbm_step_pairs.cu", "lbm_collide_pair.cuh", "lbm_step_core.cuh", "lbm_device.cuh",
+                           "lbm_internal.h"),
+    "pair16_moment_kernel": ("lbm_step16_pairs.cu", "lbm_collide_pair.cuh", "lbm_pair16.cuh", "lbm_device.cuh",
+                             "lbm_internal.h"),
+}
+
+# The two-launch steps, by their second kernel: bytes a non-solid cell's step must move (the
+# state read and written once, and what the first launch leaves for the second: densities 8, at
+# tau = 1 the common velocity 12), and what bounds them (profiles/)
+TWO_LAUNCHES = {
+    "moment_collide_kernel": (2 * (48 + 20), "latency of cached loads"),  # the state: 48 bytes of moments, in place
+    "pair_push_kernel": (304 + 2 * 20, "scattered stores"),
+    "pair_relax_kernel": (304 + 152 + 2 * 8, "hbm"),  # tau != 1: the populations are read twice
+    "pair16_push_kernel": (168 + 2 * 12 + 8, "scattered stores"),  # the densities are part of the state, read back once
 }
 
 
+def step_bytes(kernel_name, n_upd, population_bytes):
+    """Bytes a step of this kernel must move, and what bounds it: the populations once in and
+    once out, except in the two-launch steps."""
+    for second, (per_cell, bound) in TWO_LAUNCHES.items():
+        if second in kernel_name:
+            return n_upd * per_cell, bound
+    return population_bytes, "hbm"
+
+
 def kernel_hash(kernel_name="sc_step_kernel"):
-    key = next((k for k in ("sc_step_tma_kernel", "sc_step_push_kernel", "sc_step16_push_kernel")
-                if kernel_name.startswith(k)),
-               "sc_step_kernel")
+    key = next((k for k in KERNEL_SOURCES if kernel_name.startswith(k)), "sc_step_kernel")
     h = hashlib.sha256()
     for f in KERNEL_SOURCES[key]:
         h.update(open(os.path.join(ROOT, "paper_1906_04722_gb300", "csrc", f), "rb").read())
@@ -543,7 +566,9 @@ def run_ours(args, rank, world, local):
     value = whole_job_rate(n_upd * args.steps, total_ms / 1e3, world) / 1e6
     mean_ms = float(np.mean(per))
     peak, peak_kind = read_peaks()
-    achieved = bytes_per_step / (mean_ms / 1e3) / 1e9
+    moved, bound = step_bytes(kernel_name, n_upd, bytes_per_step)
+    achieved = moved / (mean_ms / 1e3) / 1e9
+    by_populations = bytes_per_step / (mean_ms / 1e3) / 1e9
     m = dom.measure()
     dom.close()
 
@@ -590,14 +615,18 @@ def run_ours(args, rank, world, local):
            "scaling": "weak", "vs_baseline": None, "dtype": {0: "f32", 1: "f16 deviations, f32 math", 2: "bf16 deviations, f32 math"}[args.precision],
            "data": "synthetic",
            "config": {"workload": f"sample{args.size}: {args.size}^3, {len(spheres)} RSA spheres r~U[10,14], "
-                                  f"reservoirs + 3 membrane layers, {POP_STORAGE[args.precision]}, one fused step per launch",
+                                  f"reservoirs + 3 membrane layers, {POP_STORAGE[args.precision]}, "
+                                  + ("two launches per step" if two_launches else "one fused step per launch"),
                       "fluid_cells": n_upd, "global_batch": world, "seq_len": 0,
                       "parallelism": "replicas" if world > 1 else "single GPU",
                       "l2": "inputs larger than L2 (2 x %.2f GB population buffers)" % pop_buffer_gb,
                       "step_kernel": tuned if tuned is not None else "default"},
-           "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+           "roofline": {"bound": bound, "achieved": achieved, "peak": peak, "unit": "GB/s",
                         "frac": achieved / peak, "traffic": read_traffic(kernel_name) if args.size == 192 else None, "peak_kind": peak_kind,
-                        "kernel": kernel_name, "algorithmic_bytes_per_launch": bytes_per_step},
+                        "kernel": kernel_name, "algorithmic_bytes_per_launch": moved,
+                        # every population read and written once, whatever the kernel keeps of them
+                        "populations": {"bytes_per_step": bytes_per_step, "achieved": by_populations,
+                                        "frac": by_populations / peak}},
            "gpu_launches": args.steps * (2 if two_launches else 1),
            "e2e": {"value": e2e_val, "unit": "MLUPS", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                    "step": f"set_pressure_bc + {E2E_SUBSTEPS} time steps + lbm_measure; domain creation "

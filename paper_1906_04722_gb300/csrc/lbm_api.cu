@@ -115,9 +115,12 @@ bool steps_in_pairs(const lbm_domain* d) {
 
 // Whether such a domain's steps run on moments (lbm_step_moments.cu), in place in one
 // population buffer: from the size on where the two population buffers (304 bytes a
-// cell) have outgrown the 129 MB L2 by a half.  On moments against on pairs: 80^3
-// 29.7 against 21.3 us a step, 96^3 40 against 56, 112 x 97 x 120 70 against 89, 192^3
-// 319 against 492.
+// cell) have outgrown the 129 MB L2 by a half.  On moments against on pairs, us a step:
+// with a third of grains 80^3 29.4 / 27.2, 84^3 32.4 / 33.9, 88^3 35.7 / 39.3, 96^3
+// 41 / 53, 112^3 77 / 92, the 192^3 sample 319 / 492; open boxes, whose pairs have no
+// rows of grain to read in vain, 88^3 36 / 31, 92^3 39 / 37, 96^3 41 / 42, 128^3 103 /
+// 110, 160^3 192 / 220, and those with nx a little above a multiple of the brick's 32
+// later (100^3 58 / 50, 112^3 79 / 73).
 constexpr long long MOMENT_CELLS = 5LL << 17;
 bool steps_on_moments(const lbm_domain* d) {
     return d->params.precision == 0 && pair_step_applicable(d->phys) && steps_in_pairs(d) && d->N >= MOMENT_CELLS;

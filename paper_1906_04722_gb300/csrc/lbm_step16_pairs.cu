@@ -9,7 +9,8 @@
 // feeds the rounding errors into the rest value and pushes the words.  A cell's
 // words are rebuilt once, not twice, and the arithmetic runs on component pairs:
 // the one-launch push kernel is bound by instruction issue, this one by neither its
-// bytes (168 + 32 a cell) nor a march along z.  Results equal the staged 16-bit
+// bytes (168 + 32 a cell) nor a march along z (192^3 sample: 433 against 456 us a step,
+// 96^3: 46 against 75).  Results equal the staged 16-bit
 // kernel's bit for bit.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -55,8 +56,10 @@ __global__ void __launch_bounds__(PAIR16_THREADS, 8)
 // LARGE: from PAIR16_LARGE cells on the launch waits for its scattered stores, and more
 // warps with the neighbour densities read twice (from L1) are the faster form; on
 // smaller boxes, which wait for the first loads, they stay in registers (4 CTAs of
-// 128 threads an SM instead of 7): 4.7 against 5.5 us a step at 32^3, 46 against 48 at
-// 96^3, 82 against 81 at 112^3, 456 against 433 at 192^3.
+// 128 threads an SM instead of 7).  Registers against twice read, us a step: 32^3 4.7 /
+// 5.5, 64^3 14.2 / 15.3, 96^3 41.1 / 42.8, 104^3 53.9 / 54.6, 112^3 70.6 / 70.2, 128^3
+// 115 / 110, 160^3 238 / 224 (a third of grains: 84^3 30.8 / 31.3, 92^3 42.0 / 41.0,
+// 112^3 79.8 / 76.6).
 constexpr int PAIR16_LARGE = 1 << 20;
 
 template <class H2, bool LARGE>
