@@ -6,13 +6,13 @@
 // Every layer is a GEMM on the fifth-generation tensor cores: one thread per CTA
 // issues tcgen05.mma (BF16 or FP16 operands rounded from FP32 master values while
 // the tiles are staged in shared memory, FP32 accumulation in tensor memory), and
-// the four warps read the accumulator back with tcgen05.ld for the epilogue, which
+// eight warps read the accumulator back with tcgen05.ld for the epilogue, which
 // adds the bias, applies ReLU or the ReLU-derivative mask and writes rows through
 // shared memory.  Operands are described by strides, so the forward pass (H W^T),
-// the input gradient (dZ W) and the weight gradient (dZ^T H) share one kernel, and
-// a third grid dimension runs all ensemble members of a layer in one launch.
-// Mean squared error, bias gradients, Adam and the ensemble statistics are
-// elementwise kernels.
+// the input gradient (dZ W) and the weight gradient (dZ^T H) share one tile routine;
+// the latter two and the bias gradients of a layer are one launch, and a grid
+// dimension runs all ensemble members of a layer.  Mean squared error, Adam and the
+// ensemble statistics are elementwise kernels.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -37,7 +37,7 @@ namespace {
 // 256 takes a hidden layer's whole width.  What bounded both was the staging: 4-byte
 // loads, eight in flight, and 2-byte stores.  With 16-byte loads of a whole chunk in
 // flight and 16-byte stores: a training layer forward (5 members) 26.5 -> 8.2 us,
-// backward (three launches, now one) 63 -> 12 us; an inference layer of 16384 rows
+// backward (three launches, now one) 63 -> 12 us; an inference layer of 13107 rows
 // 110 -> 51 us.
 constexpr int TM = 128, TK = 64, GEMM_THREADS = 256;
 constexpr int TN_SMALL = 32, TN_LARGE = 256;
