@@ -60,7 +60,8 @@ inline void touch_pages(void* p, size_t bytes) {
         for (int i = 0; i < pieces; ++i) {
             const size_t last = (size_t)p + std::min(bytes, (size_t)(i + 1) * PIECE) - 1;
             unsigned char present = 0;
-            if (mincore(reinterpret_cast<void*>(last / page * page), page, &present) != 0 || !(present & 1))
+            // (it fails where nothing is mapped, a device address for instance: the copy's to refuse)
+            if (mincore(reinterpret_cast<void*>(last / page * page), page, &present) == 0 && !(present & 1))
                 absent.push_back(i);
         }
     } catch (...) {
