@@ -365,7 +365,7 @@ int run_steps(lbm_domain* d, int n) {
     // throat's ladder of 20 x 25 two-launch steps is bound by the launches of single
     // steps: 5.06 -> 3.29 ms.
     for (int size = 0; size < 2 && !captured; ++size) {
-        if (size == 1 && (n < GRAPH_STEPS[1] || ++d->short_runs <= 3)) break;
+        if (size == 1 && (n < GRAPH_STEPS[1] || (d->short_runs < 4 && ++d->short_runs < 4))) break;
         while (n >= GRAPH_STEPS[size]) {
             if (!d->graph[d->cur][size])
                 if (int rc = capture_graph(d, d->cur, size)) return rc;
