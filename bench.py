@@ -191,6 +191,12 @@ def step_bytes(kernel_name, n_upd, population_bytes):
     return population_bytes, "hbm"
 
 
+def on_moments(box):
+    """Whether the two-launch FP32 step at tau = 1 runs on moments in this box: large boxes whose
+    rows fill five eighths of the warps that take them."""
+    return math.prod(box) >= 5 << 17 and 5 * (-(-box[0] // 32) * 32) <= 8 * box[0]
+
+
 def kernel_hash(kernel_name="sc_step_kernel"):
     key = next((k for k in KERNEL_SOURCES if kernel_name.startswith(k)), "sc_step_kernel")
     h = hashlib.sha256()
@@ -528,7 +534,7 @@ def run_ours(args, rank, world, local):
     elif two_launches and not tau1:
         kernel_name = "pair_moment_kernel + pair_relax_kernel (one step)"
     elif two_launches:
-        kernel_name = ("moment_gather_kernel + moment_collide_kernel" if box[0] * box[1] * box[2] >= 5 << 17
+        kernel_name = ("moment_gather_kernel + moment_collide_kernel" if on_moments(box)
                        else "pair_moment_kernel + pair_push_kernel") + " (one step)"
     elif args.precision and kind == lbm.KERNEL_PUSH:
         rows, stages, ctas = lbm.PUSH16_SHAPE_TABLE[tuned["shape"]][:3]

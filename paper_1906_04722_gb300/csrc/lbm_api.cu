@@ -115,15 +115,20 @@ bool steps_in_pairs(const lbm_domain* d) {
 
 // Whether such a domain's steps run on moments (lbm_step_moments.cu), in place in one
 // population buffer: from the size on where the two population buffers (304 bytes a
-// cell) have outgrown the 129 MB L2 by a half.  On moments against on pairs, us a step:
-// with a third of grains 80^3 29.4 / 27.2, 84^3 32.4 / 33.9, 88^3 35.7 / 39.3, 96^3
-// 41 / 53, 112^3 77 / 92, the 192^3 sample 319 / 492; open boxes, whose pairs have no
-// rows of grain to read in vain, 88^3 36 / 31, 92^3 39 / 37, 96^3 41 / 42, 128^3 103 /
-// 110, 160^3 192 / 220, and those with nx a little above a multiple of the brick's 32
-// later (100^3 58 / 50, 112^3 79 / 73).
+// cell) have outgrown the 129 MB L2 by a half, in boxes whose rows fill five eighths of
+// the warps that take them (steps and read-outs cost 45 to 49 ps a lane; the pairs, of
+// whole warps whatever the box, 46 to 54 ps a cell and with a third of grains 57 to 70).
+// On moments against on pairs, us a step: with a third of grains 80^3 29.4 / 27.2, 84^3
+// 32.4 / 33.9, 88^3 35.7 / 39.3, 96^3 41 / 53, 112^3 77 / 92, the 192^3 sample 319 /
+// 492, and rows of 47, 40 and 33 cells (x 180 x 180) 95 / 113, 89 / 86, 81 / 77; open
+// boxes, whose pairs have no rows of grain to read in vain, 88^3 36 / 31, 92^3 39 / 37,
+// 96^3 41 / 42, 100^3 58 / 50, 128^3 103 / 110, 160^3 192 / 220, 33 x 180 x 180 86 / 65,
+// 5 x 400 x 400 192 / 69, 1 x 1000 x 1000 1172 / 194 (and lbm_measure 951 / 101), but
+// 1000 x 1000 x 1 47 / 49.
 constexpr long long MOMENT_CELLS = 5LL << 17;
 bool steps_on_moments(const lbm_domain* d) {
-    return d->params.precision == 0 && pair_step_applicable(d->phys) && steps_in_pairs(d) && d->N >= MOMENT_CELLS;
+    return d->params.precision == 0 && pair_step_applicable(d->phys) && steps_in_pairs(d) && d->N >= MOMENT_CELLS &&
+           5 * ((d->geom.nx + MOMENT_ROW - 1) / MOMENT_ROW * MOMENT_ROW) <= 8 * d->geom.nx;
 }
 
 // One step from buffer `cur` to buffer cur ^ 1 (on moments: in place) on stream s.

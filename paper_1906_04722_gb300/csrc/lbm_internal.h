@@ -162,6 +162,7 @@ cudaError_t launch_pair_moments(float* F, float2* rho2, const uint32_t* nbr, con
 // tau = 1 in both components on moments, in place in one population buffer
 // (lbm_step_moments.cu); the first step starts from the paired push layout F (left
 // with intermediate values) and builds the moments in `buffer`
+constexpr int MOMENT_ROW = 32;  // cells of a row that one warp of its kernels takes
 cudaError_t launch_step_moments(float* buffer, const uint32_t* nbr, const uint32_t* nbr_nw, const uint32_t* adh,
                                 const Geom& g, const Phys& p, cudaStream_t s);
 cudaError_t launch_first_moments(float* F, float2* rho2, float* buffer, const uint32_t* nbr, const uint32_t* adh,

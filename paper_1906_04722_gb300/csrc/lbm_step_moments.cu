@@ -28,7 +28,7 @@ namespace lbmk {
 
 namespace {
 
-constexpr int MX = 32, MY = 4, MZ = 2, MT = MX * MY * MZ;
+constexpr int MX = MOMENT_ROW, MY = 4, MZ = 2, MT = MX * MY * MZ;
 
 // Arrays of the state in a population buffer, `plane` pairs apart.
 struct Moments {
