@@ -468,6 +468,9 @@ __global__ void rest_density_kernel(const uint8_t* __restrict__ mask, float* __r
 // Densities between the host's doubles and the device's floats, converted on the
 // device piece by piece (a host loop over the 192^3 sample's 14 M values took 8 ms).
 constexpr long long CONVERT_PIECE = 4LL << 20;  // doubles
+// Small fields are converted by the host, with one wait and no second launch: 16^3 34 us
+// against 43, 24^3 42 against 45, 28^3 47 against 44, 32^3 55 against 46.
+constexpr long long HOST_CONVERT = 1LL << 15;  // values
 __global__ void to_float_kernel(const double* __restrict__ in, float* __restrict__ out, long long n) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         out[i] = (float)in[i];
@@ -847,6 +850,13 @@ int lbm_get_density(lbm_domain* d, double* rho_out) {
                                       d->stream));
         }
         const long long total = 2 * d->N;
+        if (total <= HOST_CONVERT) {
+            std::vector<float> tmp((size_t)total);
+            LBM_CUDA(cudaMemcpyAsync(tmp.data(), d->d_rho, sizeof(float) * total, cudaMemcpyDeviceToHost, d->stream));
+            if (int rc = wait_domain(d)) return rc;
+            std::copy(tmp.begin(), tmp.end(), rho_out);
+            return LBM_OK;
+        }
         auto convert = [&](long long i) {  // the piece from value i on
             to_double_kernel<<<1216, 256, 0, d->stream>>>(d->d_rho + i, d->d_convert, std::min(CONVERT_PIECE, total - i));
             return cudaGetLastError();

@@ -114,3 +114,19 @@ def test_a_failed_read_out_leaves_the_array_as_it_was(lbm, call, precision):
     assert read() == 0
     want = d.density() if call == "density" else d.state()[0]
     assert np.array_equal(out, want.ravel())
+
+
+@pytest.mark.parametrize("precision", [0, 2])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (16, 32, 32), (17, 32, 32)])
+def test_densities_converted_by_the_host_or_the_device(lbm, shape, precision):
+    """2^15 values are the largest field that the host converts."""
+    nz, ny, nx = shape
+    d = lbm.Domain(lbm.make_params(periodic=(1, 1, 1), precision=precision), None, (nx, ny, nz))
+    rho = W.droplet_densities(shape, (nx / 2, ny / 2, nz / 2), 6.0, seed=5)
+    d.set_densities(rho)
+    got = d.density()
+    want = rho.astype(np.float32)
+    assert np.allclose(got, want, rtol=1e-6, atol=0)  # the sum of 19 rest populations
+    assert np.array_equal(got, got.astype(np.float32))
+    for z, y, x in ((0, 0, 0), (nz - 1, ny - 1, nx - 1), (nz // 2, ny // 3, nx // 4)):
+        assert tuple(got[:, z, y, x]) == tuple(d.density_at(x, y, z))
