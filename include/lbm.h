@@ -632,10 +632,11 @@ int lbm_get_tile(const lbm_domain* d, int* by, int* lz, int* lead);
  * New domains use LBM_KERNEL_STAGED; as long as neither a kernel nor a shape has
  * been chosen, an FP32 domain, and a 16-bit domain with tau = 1 in both
  * components, steps in the two launches of LBM_KERNEL_SPLIT, with the same bits
- * (lbm_autotune times every kind that applies on the domain).  All give the same results up to rounding (not bit for bit:
- * the TMA kernel folds omega w_k into its equilibrium constants).  LBM_ERR_ARG
- * for an unknown kind, LBM_ERR_STATE when the kernel does not apply to the
- * domain.  lbm_set_tile switches the domain to LBM_KERNEL_STAGED. */
+ * (lbm_autotune times every kind that applies on the domain).  All give the same
+ * results up to rounding (not bit for bit: the TMA kernel folds omega w_k into its
+ * equilibrium constants).  LBM_ERR_ARG for an unknown kind, LBM_ERR_STATE when the
+ * kernel does not apply to the domain.  lbm_set_tile switches the domain to
+ * LBM_KERNEL_STAGED. */
 #define LBM_KERNEL_STAGED 0
 #define LBM_KERNEL_TMA 1
 #define LBM_KERNEL_SPLIT 2
